@@ -283,6 +283,8 @@ hq_status hq_apply_blocks(void *state, int n, hq_dtype dt, const hq_gate *gates,
     }
     if (engine == HQ_ENGINE_TC_F16 || engine == HQ_ENGINE_TC_BF16)
         return launch_tc_blocks(state, n, gates, G, tc_min_k, engine == HQ_ENGINE_TC_BF16, (cudaStream_t)stream);
+    if (engine == HQ_ENGINE_AUTO || engine == HQ_ENGINE_CUDA_CORE)
+        return launch_gate_list(state, n, dt, gates, G, engine, (cudaStream_t)stream);
     for (int g = 0; g < G; ++g) {
         st = launch_gate(state, n, dt, gates[g].k, gates[g].qubits, gates[g].matrix, 1, engine, (cudaStream_t)stream);
         if (st != HQ_OK) return st;

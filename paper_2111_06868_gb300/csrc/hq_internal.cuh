@@ -222,6 +222,9 @@ hq_status launch_upload(void *state, const void *host, size_t bytes, cudaStream_
 hq_status launch_init(void *state, int n, hq_dtype dt, const char *tokens, int64_t nstates, cudaStream_t s);
 hq_status launch_gate(void *state, int n, hq_dtype dt, int k, const int *qubits, const double *matrix,
                       int64_t nstates, int engine, cudaStream_t s);
+// G gates in order on the exact engines (HQ_ENGINE_AUTO, HQ_ENGINE_CUDA_CORE),
+// narrow ones many at a time (k_runs.cu), the others through launch_gate
+hq_status launch_gate_list(void *state, int n, hq_dtype dt, const hq_gate *gates, int G, int engine, cudaStream_t s);
 bool is_diagonal(int k, const double *matrix);
 // exactly one nonzero per row and column; perm[r] = column of row r (may be NULL)
 bool is_monomial(int k, const double *matrix, int *perm);
