@@ -12,7 +12,7 @@
 //     parameter space (uniform constant-bank operands of the FMAs), and streams
 //     the tile back.  An XOR swizzle of the shared-memory index keeps both the
 //     linear copy and the strided group access free of bank conflicts.
-//     complex64 runs k_gather_pipe, the same with two tile buffers: the
+//     complex64 runs k_gather_pipe (K <= 2) or k_gather_pair, with two tile buffers: the
 //     cp.async copy of the next tile is in flight while the current one is
 //     multiplied and stored.
 //   * k_diag<R, K>: diagonal gates (CZ, RZ, CPHASE and fused diagonal blocks)
@@ -236,17 +236,12 @@ template <typename R, int K> struct MatParam {
 
 constexpr int kThreads = 256;
 
-// Rows of M one thread accumulates, and threads sharing one group.  K <= 2,
-// and K = 3 in complex64: one thread owns a whole group and writes it back in
-// place at once (the pipelined complex64 kernel runs 3 CTAs per SM, which
-// leaves room for the 8 inputs and 8 accumulators).  Otherwise (K = 4, and
-// K = 3 in complex128): a warp takes 32 groups and one 4-row chunk of M (so
-// every lane reads the same, compile-time-indexed M entries: constant-bank
-// operands), holds its accumulators across a barrier, then writes.
-template <typename R, int K> __host__ __device__ constexpr int gather_rows()
-{
-    return K <= 2 ? (1 << K) : (K == 3 && sizeof(R) == 4) ? 8 : 4;
-}
+// Rows of M one thread accumulates, and threads sharing one group.  K <= 2: one
+// thread owns a whole group and writes it back in place at once.  K = 3, 4
+// (complex128): a warp takes 32 groups and one 4-row chunk of M (so every lane
+// reads the same, compile-time-indexed M entries: constant-bank operands),
+// holds its accumulators across a barrier, then writes.
+template <typename R, int K> __host__ __device__ constexpr int gather_rows() { return K <= 2 ? (1 << K) : 4; }
 template <typename R, int K> __host__ __device__ constexpr int gather_tpg() { return (1 << K) / gather_rows<R, K>(); }
 // work items (group x chunk) per thread for a full tile of 2^LB amplitudes
 template <typename R, int K, int LB> __host__ __device__ constexpr int gather_items()
@@ -268,12 +263,6 @@ __device__ __forceinline__ void gather_rows_acc(const MatParam<R, K> &m, const t
         for (int rr = 0; rr < NR; ++rr) cmac(acc[rr], m.a[R0 + rr][c], v);
     }
 }
-
-// Tile of 2^12 complex64 (32 KB per buffer, 3 CTAs per SM) for K = 3; 2^11
-// (16 KB, more CTAs) otherwise (n=30, GB/s at 12 / 11 bits: K=1 6455-6570 /
-// 6478-6596, K=2 6259-6458 / 6327-6547, K=3 5386-5704 / 5124-5810, K=4
-// 2144-2175 / 2404-2598 with 4-row chunks).
-template <int K> constexpr int gather_pipe_tile_bits() { return K == 3 ? 12 : 11; }
 
 // One tile in shared memory multiplied in place (every group of 2^K
 // amplitudes by the matrix); ends with a barrier.
@@ -350,6 +339,7 @@ __global__ void __launch_bounds__(kThreads) k_gather(const TileGeom g, const Mat
 // whose swizzle is odd (the two amplitudes trade places) as two 8-byte
 // copies.
 // ----------------------------------------------------------------------------
+
 __device__ __forceinline__ void tile_load_async(const TileGeom &g, const int64_t *runoff,
                                                 const float2 *__restrict__ base, float2 *tile)
 {
@@ -365,7 +355,6 @@ __device__ __forceinline__ void tile_load_async(const TileGeom &g, const int64_t
         }
     }
 }
-
 
 __device__ __forceinline__ void tile_store_r(const TileGeom &g, const int64_t *runoff, float2 *__restrict__ base,
                                              const float2 *tile)
@@ -413,61 +402,170 @@ __device__ __forceinline__ void tiles_pipelined(const TileGeom &g, float2 *__res
     cp_async_wait<0>();
 }
 
-// K = 4 in complex64: as gather_tile's chunked form, with the matrix read
-// from shared memory (every lane of a warp reads the same entry: a
-// broadcast) at a row offset known only at run time, so that one copy of the
-// unrolled 4 x 16 multiply-add body serves all four row chunks (four
-// constant-operand copies of it did not stay in the instruction cache).
-// (Packed FMAs with the entries stored as (Re, Re, -Im, Im) took 20 % longer:
-// one 16-byte shared load per complex multiply-add.)
-template <int LB>
-__device__ __forceinline__ void gather_tile_k4_sh(const TileGeom &g, const float2 (*msh)[16], float2 *tile)
+// The same for kernels that the issue slots bound, tiles of 2^g.L <= 2^LB
+// amplitudes and TH >= 128 threads: a thread's copies lie 2 TH amplitudes
+// apart, above the bits the swizzle reads, so each address is the thread's
+// first one plus an offset that all threads share (from shared memory in the
+// state, an immediate in the tile).  Per-copy addresses cost the K = 4 kernel
+// 10 % (n = 28: 0.96 against 0.87 ms); for the HBM-bound kernels above the plain loops
+// are the faster form (K = 1: 0.675 against 0.695 ms).
+template <int LB, int TH, typename Op>
+__device__ __forceinline__ void tiles_pipelined_lean(const TileGeom &g, float2 *__restrict__ state, Op op)
 {
-    constexpr int K = 4, NR = gather_rows<float, K>(), TPG = gather_tpg<float, K>(), NI = gather_items<float, K, LB>();
-    const int ngroups = (1 << g.L) >> K;
-    float2 acc[NI][NR];
-    int ibs[NI], chunk[NI];
-#pragma unroll
-    for (int it = 0; it < NI; ++it) {
-        const int w = it * kThreads + threadIdx.x;
-        const int wi = w >> 5;
-        chunk[it] = wi % TPG;
-        const int grp = (wi / TPG) * 32 + (w & 31);
-        ibs[it] = -1;
-#pragma unroll
-        for (int rr = 0; rr < NR; ++rr) acc[it][rr].x = acc[it][rr].y = 0;
-        if (grp < ngroups) {
-            ibs[it] = group_base<K>(g, grp);
-            const float2 (*mr)[16] = msh + chunk[it] * NR;
-#pragma unroll
-            for (int c = 0; c < (1 << K); ++c) {
-                const float2 v = tile[swz<float>(ibs[it] + g.toff[c])];
-#pragma unroll
-                for (int rr = 0; rr < NR; ++rr) cmac(acc[it][rr], mr[rr][c], v);
-            }
-        }
+    static_assert(TH >= 128 && (2 * TH) <= (1 << LB), "");
+    constexpr int STEP = 2 * TH, NC = (1 << LB) / STEP;
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    __shared__ int64_t s_k[NC];  // flat offset of a thread's k-th copy from its first
+    float2 *const buf = reinterpret_cast<float2 *>(smem_raw);
+    const int TS = 1 << g.L, cmask = (1 << g.c) - 1;
+    const int first = int(threadIdx.x) * 2, f = (first >> 4) & 15;
+    const bool copier = first < TS;
+    if (threadIdx.x < NC && int(threadIdx.x) * STEP < TS) {
+        const int i = int(threadIdx.x) * STEP;
+        s_k[threadIdx.x] = g.runoff[i >> g.c] + (i & cmask);
     }
+    const int64_t off = copier ? g.runoff[first >> g.c] + (first & cmask) : 0;
     __syncthreads();
+    const bool full = g.L == LB;  // (smaller only for states of fewer than LB qubits: one tile)
+    // both loops free of conditions when the tile is full: the loads of all copies overlap
+    auto load = [&](int64_t t, float2 *to) {
+        const float2 *const src = state + tile_base(g, t) + off;
+        auto copy = [&](int k) {
+            if (f & 1) {
+                cp_async8(to + (first ^ f) + k * STEP, src + s_k[k]);
+                cp_async8(to + ((first + 1) ^ f) + k * STEP, src + s_k[k] + 1);
+            } else {
+                cp_async16(to + (first ^ f) + k * STEP, src + s_k[k]);
+            }
+        };
+        if (full) {
 #pragma unroll
-    for (int it = 0; it < NI; ++it)
-        if (ibs[it] >= 0)
+            for (int k = 0; k < NC; ++k) copy(k);
+        } else if (copier) {
+            for (int k = 0; k * STEP < TS; ++k) copy(k);
+        }
+    };
+    auto store = [&](int64_t t, const float2 *from) {
+        float2 *const dst = state + tile_base(g, t) + off;
+        auto copy = [&](int k) {
+            const float4 w = *reinterpret_cast<const float4 *>(from + ((first ^ f) & ~1) + k * STEP);
+            *reinterpret_cast<float4 *>(dst + s_k[k]) = (f & 1) ? make_float4(w.z, w.w, w.x, w.y) : w;
+        };
+        if (full) {
 #pragma unroll
-            for (int rr = 0; rr < NR; ++rr) tile[swz<float>(ibs[it] + g.toff[chunk[it] * NR + rr])] = acc[it][rr];
-    __syncthreads();
+            for (int k = 0; k < NC; ++k) copy(k);
+        } else if (copier) {
+            for (int k = 0; k * STEP < TS; ++k) copy(k);
+        }
+    };
+    int64_t t = blockIdx.x;
+    if (t >= g.total_tiles) return;
+    int b = 0;
+    load(t, buf);
+    cp_async_commit();
+    for (; t < g.total_tiles; t += gridDim.x) {
+        const int64_t tn = t + gridDim.x;
+        float2 *const cur = buf + b * TS;
+        b ^= 1;
+        // the other buffer was last read by the store of tile t - grid, before the barrier that ended it
+        if (tn < g.total_tiles) load(tn, buf + b * TS);
+        cp_async_commit();   // possibly empty: every thread waits on the same group count
+        cp_async_wait<1>();  // this thread's copies of tile t have landed
+        __syncthreads();     // ... and everyone else's
+        op(cur);
+        store(t, cur);
+        __syncthreads();
+    }
+    cp_async_wait<0>();
 }
 
+// K = 3, 4 in complex64: one thread takes a whole group (its amplitudes in
+// registers as (re, im) pairs) and writes each row of the product as soon as
+// it has it -- nobody else touches the group, so there is no barrier and no
+// accumulator beyond the current row's.  A row is two sums of packed FMAs,
+//   A = sum_c Re(m_rc) (x_c, y_c),  B = sum_c Im(m_rc) (x_c, y_c),
+//   out_r = (A.x - B.y, A.y + B.x),
+// which need no swapped copies of the inputs; the matrix lies in the parameter
+// block with both parts duplicated ((re, re, im, im): constant-bank operands
+// of the packed FMAs, no load).  K = 4 is 64 FMAs per amplitude: 0.46 ms at
+// n = 28 on the FP32 pipes against 0.63 ms of HBM time.
+// n = 28, targets on qubits 0..3 / 27..24 / 3, 12, 20, 26:
+//   K = 4   4-row chunks per warp, matrix in shared memory   1.31 / 1.23 / 1.41 ms
+//           this                                             0.86 / 0.84 / 0.88 ms (5000 GB/s)
+//   K = 3   8 rows per thread, scalar constant operands      0.80 / 0.76 / 0.79 ms (targets 0..2 / 27..25 / 3, 12, 20)
+//           this                                             0.71 / 0.69 / 0.71 ms (6030 GB/s)
+// Slower for K = 4: scalar FMAs with constant operands by 14 %, the matrix from shared memory (16-byte broadcasts)
+// with two groups per thread 20 %, 4 rows x 4 groups per thread 27 %, 2^12 tiles with 256 threads 8 % (fewer CTAs
+// out of step), five CTAs per SM at 96 registers 3 %.
+template <int K> struct PairMatParam {
+    ulonglong2 a[1 << K][1 << K];  // (re, re), (im, im)
+    int off[1 << K];               // swizzled byte offset of local index r in a tile
+};
+
+__device__ __forceinline__ unsigned long long pair_mul(unsigned long long x, unsigned long long y)
+{
+    unsigned long long d;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(x), "l"(y));
+    return d;
+}
+__device__ __forceinline__ unsigned long long pair_fma(unsigned long long x, unsigned long long y,
+                                                       unsigned long long z)
+{
+    unsigned long long d;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(x), "l"(y), "l"(z));
+    return d;
+}
+__device__ __forceinline__ float2 pair_split(unsigned long long v)
+{
+    float2 h;
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(h.x), "=f"(h.y) : "l"(v));
+    return h;
+}
+
+constexpr int kPairTileBits = 11, kPairThreads = 128;
+
+template <int K>
+__global__ void __launch_bounds__(kPairThreads, 4) k_gather_pair(const __grid_constant__ TileGeom g,
+                                                                 const __grid_constant__ PairMatParam<K> p,
+                                                                 float2 *__restrict__ state)
+{
+    constexpr int D = 1 << K;
+    auto op = [&](float2 *tile) {
+        char *const tb = reinterpret_cast<char *>(tile);
+        const int ngroups = (1 << g.L) >> K;
+#pragma unroll 1
+        for (int grp = threadIdx.x; grp < ngroups; grp += kPairThreads) {
+            // the swizzle is linear over XOR and a group's base has no target bit: slot(base | target bits) =
+            // slot(base) ^ off[r]
+            const int a0 = swz<float>(group_base<K>(g, grp)) * int(sizeof(float2));
+            unsigned long long v[D];
+#pragma unroll
+            for (int c = 0; c < D; ++c) v[c] = *reinterpret_cast<const unsigned long long *>(tb + (a0 ^ p.off[c]));
+#pragma unroll
+            for (int r = 0; r < D; ++r) {
+                unsigned long long A = pair_mul(p.a[r][0].x, v[0]), B = pair_mul(p.a[r][0].y, v[0]);
+#pragma unroll
+                for (int c = 1; c < D; ++c) {
+                    A = pair_fma(p.a[r][c].x, v[c], A);
+                    B = pair_fma(p.a[r][c].y, v[c], B);
+                }
+                const float2 x = pair_split(A), y = pair_split(B);
+                *reinterpret_cast<float2 *>(tb + (a0 ^ p.off[r])) = make_float2(x.x - y.y, x.y + y.x);
+            }
+        }
+        __syncthreads();
+    };
+    // K = 3 is near HBM (0.71 ms; lean 0.72), K = 4 is issue-bound (lean 0.87; plain 0.96)
+    if constexpr (K == 3) tiles_pipelined(g, state, op);
+    else tiles_pipelined_lean<kPairTileBits, kPairThreads>(g, state, op);
+}
+
+// K = 1, 2 in complex64: bound by HBM with plain FMAs
 template <int K>
 __global__ void __launch_bounds__(kThreads) k_gather_pipe(const TileGeom g, const MatParam<float, K> m,
                                                           float2 *__restrict__ state)
 {
-    if constexpr (K == 4) {
-        __shared__ float2 msh[16][16];
-        for (int i = threadIdx.x; i < 256; i += blockDim.x) msh[i >> 4][i & 15] = m.a[i >> 4][i & 15];
-        // (tiles_pipelined's first barrier orders these stores before the reads)
-        tiles_pipelined(g, state, [&](float2 *tile) { gather_tile_k4_sh<gather_pipe_tile_bits<K>()>(g, msh, tile); });
-    } else {
-        tiles_pipelined(g, state, [&](float2 *tile) { gather_tile<float, K, gather_pipe_tile_bits<K>()>(g, m, tile); });
-    }
+    tiles_pipelined(g, state, [&](float2 *tile) { gather_tile<float, K, 11>(g, m, tile); });
 }
 
 // ----------------------------------------------------------------------------
@@ -807,21 +905,37 @@ static hq_status run_gather(void *state, int n, const int *qubits, const double 
             m.a[r][c].x = R(mat[2 * (r * (1 << K) + c)]);
             m.a[r][c].y = R(mat[2 * (r * (1 << K) + c) + 1]);
         }
-    if constexpr (sizeof(R) == 4) {
-        // complex64: the FP32 work of a tile is short next to its HBM time, so
-        // the next tile's load runs under it (two buffers per CTA)
-        make_geom(g, n, K, qubits, std::min(n, gather_pipe_tile_bits<K>()), nstates);
+    // complex64: the next tile's load in flight under the current one (two buffers per CTA)
+    if constexpr (sizeof(R) == 4 && K >= 3) {
+        make_geom(g, n, K, qubits, std::min(n, kPairTileBits), nstates);
+        PairMatParam<K> p;
+        for (int r = 0; r < (1 << K); ++r) {
+            p.off[r] = (g.toff[r] ^ ((g.toff[r] >> 4) & 15)) * int(sizeof(float2));
+            for (int c = 0; c < (1 << K); ++c) {
+                const float2 re = make_float2(m.a[r][c].x, m.a[r][c].x), im = make_float2(m.a[r][c].y, m.a[r][c].y);
+                std::memcpy(&p.a[r][c].x, &re, 8);
+                std::memcpy(&p.a[r][c].y, &im, 8);
+            }
+        }
+        const size_t smem = size_t(2 * sizeof(float2)) << g.L;
+        const void *fn = (const void *)k_gather_pair<K>;
+        const int grid = grid_for(fn, kPairThreads, smem, g.total_tiles);
+        k_gather_pair<K><<<grid, kPairThreads, smem, s>>>(g, p, (float2 *)state);
+        return cuda_status("k_gather_pair", cudaGetLastError());
+    } else if constexpr (sizeof(R) == 4) {
+        make_geom(g, n, K, qubits, std::min(n, 11), nstates);
         const size_t smem = size_t(2 * sizeof(float2)) << g.L;
         const void *fn = (const void *)k_gather_pipe<K>;
         const int grid = grid_for(fn, kThreads, smem, g.total_tiles);
         k_gather_pipe<K><<<grid, kThreads, smem, s>>>(g, m, (float2 *)state);
         return cuda_status("k_gather_pipe", cudaGetLastError());
-    }
+    } else {
     const size_t smem = size_t(sizeof(typename C2<R>::type)) << g.L;
     const void *fn = (const void *)k_gather<R, K>;
     const int grid = grid_for(fn, kThreads, smem, g.total_tiles);
     k_gather<R, K><<<grid, kThreads, smem, s>>>(g, m, (typename C2<R>::type *)state);
     return cuda_status("k_gather", cudaGetLastError());
+    }
 }
 
 template <typename R, int K>
