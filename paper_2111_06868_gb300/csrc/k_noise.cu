@@ -426,6 +426,408 @@ static hq_status sample_on_device(void *state, int n, const int *qubits, PickArg
     return cuda_status("k_apply_sel", cudaGetLastError());
 }
 
+// ----------------------------------------------------------------------------
+// Windows: one or two state-dependent channels per trip through the state
+//
+// Two one-qubit channels on different qubits, with nothing but absorbed gates
+// between them, need one joint reduced density matrix: the first channel's
+// probabilities come from its partial trace, the second's from the same matrix
+// after the operator picked for the first,
+//   rho2[b][b'] = sum_cc' (M^dag M)[c'][c] rho[(c, b)][(c', b')].
+// k_window picks (every CTA for itself, from the partial sums of the launch
+// before: no extra launch, no CTA waits for another), applies both operators
+// to its groups and, from the amplitudes it writes, sums the reduced density
+// matrix of the next window's qubits.  So a channel costs half of one read and
+// write of the state instead of a read, a one-CTA pick and a read and write.
+// A thread holds 16 amplitudes: all values of this window's two qubits and of
+// the next one's (a qubit that a window lacks is replaced by any other bit).
+// Bound: HBM (two channels at n = 24: 268 MB, 40 us at the copy bandwidth), with
+// about 5 us of FP64 latency per launch for the pick; complex128 the FP64 pipe.
+// ----------------------------------------------------------------------------
+constexpr int kWindowRow = 20;  // doubles per CTA: 10 complex entries of the upper triangle
+struct WindowParam {
+    int64_t off[16];   // flat offset of local index 4 a + b (a: this window's qubits, b: the next one's; first qubit
+                       // most significant)
+    int fixed[4];      // the four bits, ascending
+    int free_bits;     // n - 4
+    int na, nb;        // qubits of this window (0: nothing to apply) and of the next (0: nothing to sum)
+    int nch;           // channels of this window: 2 one-qubit ones, or 1 on na qubits
+    const double *K[2], *G[2], *A[2], *u[2];  // per channel: as in PickArgs
+    int nK[2];
+    int *chosen[2];
+    int *status;
+    const double *in;  // partial sums for this window: `rows` rows of kWindowRow
+    int rows;
+    double *out;       // partial sums for the next window, one row per CTA
+};
+
+// One warp: the branch of a channel on D levels with reduced density matrix
+// rho0 (shared memory, D x D complex), its renormalised operator times the
+// absorbed gates in M (FP64, shared memory); true when that is the identity to
+// rounding.  The matrix products take one lane per entry (FP64 instructions are
+// what they cost, whatever the lanes do); the sums run in k_kraus_pick's order.
+template <int D>
+__device__ __forceinline__ bool window_pick(const double *rho0, const double *K, const double *G, const double *A,
+                                            double u, int nK, double *T, double *prob, double *M, int *chosen,
+                                            int *status, bool report)
+{
+    constexpr int DD = D * D;
+    const int lane = threadIdx.x & 31, x = (lane % DD) / D, y = lane % D;
+    double sr = 0, si = 0;
+#pragma unroll
+    for (int z = 0; z < D; ++z) {  // T = A rho0
+        const double ar = A[2 * (x * D + z)], ai = A[2 * (x * D + z) + 1];
+        const double br = rho0[2 * (z * D + y)], bi = rho0[2 * (z * D + y) + 1];
+        sr += ar * br - ai * bi;
+        si += ar * bi + ai * br;
+    }
+    __syncwarp();
+    if (lane < DD) T[2 * lane] = sr, T[2 * lane + 1] = si;
+    __syncwarp();
+    sr = si = 0;
+#pragma unroll
+    for (int z = 0; z < D; ++z) {  // rho = T A^dag
+        const double ar = T[2 * (x * D + z)], ai = T[2 * (x * D + z) + 1];
+        const double br = A[2 * (y * D + z)], bi = -A[2 * (y * D + z) + 1];
+        sr += ar * br - ai * bi;
+        si += ar * bi + ai * br;
+    }
+    __syncwarp();
+    if (lane < DD) T[2 * lane] = sr, T[2 * lane + 1] = si;
+    __syncwarp();
+    for (int i = lane; i < nK; i += 32) {  // p_i = Tr(rho K_i^dag K_i)
+        const double *g = G + size_t(i) * 2 * DD;
+        double t = 0;
+#pragma unroll
+        for (int r = 0; r < D; ++r)
+#pragma unroll
+            for (int c = 0; c < D; ++c)
+                t += T[2 * (r * D + c)] * g[2 * (c * D + r)] - T[2 * (r * D + c) + 1] * g[2 * (c * D + r) + 1];
+        prob[i] = fmax(t, 0.0);
+    }
+    __syncwarp();
+    double total = 0;
+    for (int i = 0; i < nK; ++i) total += prob[i];
+    int pick = -1;
+    double cum = 0, ppick = 0;
+    const double target = u * total;
+    for (int i = 0; i < nK; ++i) {
+        const double pi = prob[i];
+        cum += pi;
+        if (pi > 0) {
+            pick = i;
+            ppick = pi;
+            if (cum > target) break;
+        }
+    }
+    if (!(total > 0)) pick = -1;
+    double mr = x == y ? 1.0 : 0.0, mi = 0;
+    if (pick >= 0) {
+        const double sc = 1.0 / sqrt(ppick);
+        const double *Kp = K + size_t(pick) * 2 * DD;
+        mr = 0;
+#pragma unroll
+        for (int z = 0; z < D; ++z) {  // (K_pick A)[x][y] / sqrt(p_pick)
+            const double kr = Kp[2 * (x * D + z)], ki = Kp[2 * (x * D + z) + 1];
+            const double ar = A[2 * (z * D + y)], ai = A[2 * (z * D + y) + 1];
+            mr += kr * ar - ki * ai;
+            mi += kr * ai + ki * ar;
+        }
+        mr *= sc;
+        mi *= sc;
+    }
+    const double dr = mr - (x == y ? 1.0 : 0.0);
+    const bool one = dr * dr + mi * mi <= 16.0 * 2.220446049250313e-16 * 2.220446049250313e-16;
+    const bool identity = __all_sync(0xffffffffu, one);
+    if (lane < DD) M[2 * lane] = mr, M[2 * lane + 1] = mi;
+    __syncwarp();
+    if (report && lane == 0) {
+        *chosen = pick;
+        if (pick < 0) *status = 1;
+    }
+    return identity;
+}
+
+constexpr int kWindowThreads = 256;
+
+template <typename R>
+__global__ void __launch_bounds__(kWindowThreads, sizeof(R) == 4 ? 2 : 1) k_window(const __grid_constant__ WindowParam p,
+                                                              typename C2<R>::type *__restrict__ psi)
+{
+    using T2 = typename C2<R>::type;
+    __shared__ double s_part[kWindowThreads / 32][kWindowRow];
+    __shared__ double s_rho[32], s_one[32], s_T[32], s_prob[kMaxKraus], s_M[2][32];
+    __shared__ T2 s_m[2][16];
+    __shared__ int s_identity[2];
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int64_t groups = int64_t(1) << p.free_bits, stride = int64_t(gridDim.x) * blockDim.x;
+    auto spread = [&](int64_t f) {
+        int64_t x = f;
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            const int b = p.fixed[j];
+            x = ((x >> b) << (b + 1)) | (x & ((int64_t(1) << b) - 1));
+        }
+        return x;
+    };
+    T2 v[16];
+    int64_t f = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
+    // the first group's loads run under the pick
+    T2 *base = psi + (f < groups ? spread(f) : 0);
+    if (f < groups) {
+#pragma unroll
+        for (int i = 0; i < 16; ++i) v[i] = base[p.off[i]];
+    }
+    if (p.na > 0) {
+        // the CTAs' sums, in a fixed order: rows warp by warp, one column per lane
+        const int width = p.na == 1 ? 6 : kWindowRow;
+        double t = 0;
+        if (lane < width)
+            for (int r = warp; r < p.rows; r += kWindowThreads / 32) t += p.in[int64_t(r) * kWindowRow + lane];
+        if (lane < kWindowRow) s_part[warp][lane] = t;
+        __syncthreads();
+        if (warp == 0) {
+            t = 0;
+            if (lane < width)
+                for (int w = 0; w < kWindowThreads / 32; ++w) t += s_part[w][lane];
+            // upper triangle -> full matrix
+            const int D = 1 << p.na;
+            if (lane < width) {
+                int e = lane >> 1, r = 0;
+                while (e >= D - r) e -= D - r, ++r;
+                const int c = r + e, im = lane & 1;
+                s_rho[2 * (r * D + c) + im] = t;
+                if (r != c) s_rho[2 * (c * D + r) + im] = im ? -t : t;
+            }
+            __syncwarp();
+            bool id0, id1 = true;
+            const bool report = blockIdx.x == 0;
+            if (p.nch == 1) {
+                id0 = p.na == 1 ? window_pick<2>(s_rho, p.K[0], p.G[0], p.A[0], *p.u[0], p.nK[0], s_T, s_prob, s_M[0],
+                                                 p.chosen[0], p.status, report)
+                                : window_pick<4>(s_rho, p.K[0], p.G[0], p.A[0], *p.u[0], p.nK[0], s_T, s_prob, s_M[0],
+                                                 p.chosen[0], p.status, report);
+            } else {
+                // the first qubit's partial trace
+                if (lane < 8) {
+                    const int a = (lane >> 2) & 1, a2 = (lane >> 1) & 1, im = lane & 1;
+                    s_one[2 * (2 * a + a2) + im] =
+                        s_rho[2 * (4 * (2 * a) + 2 * a2) + im] + s_rho[2 * (4 * (2 * a + 1) + 2 * a2 + 1) + im];
+                }
+                __syncwarp();
+                id0 = window_pick<2>(s_one, p.K[0], p.G[0], p.A[0], *p.u[0], p.nK[0], s_T, s_prob, s_M[0], p.chosen[0],
+                                     p.status, report);
+                // Q = M^dag M, then the second qubit's matrix after the first operator
+                const int x = (lane >> 1) & 1, y = lane & 1;
+                double qr = 0, qi = 0;
+#pragma unroll
+                for (int z = 0; z < 2; ++z) {
+                    const double ar = s_M[0][2 * (2 * z + x)], ai = -s_M[0][2 * (2 * z + x) + 1];
+                    const double br = s_M[0][2 * (2 * z + y)], bi = s_M[0][2 * (2 * z + y) + 1];
+                    qr += ar * br - ai * bi;
+                    qi += ar * bi + ai * br;
+                }
+                __syncwarp();
+                if (lane < 4) s_T[2 * lane] = qr, s_T[2 * lane + 1] = qi;
+                __syncwarp();
+                double sr = 0, si = 0;
+#pragma unroll
+                for (int c = 0; c < 2; ++c)
+#pragma unroll
+                    for (int c2 = 0; c2 < 2; ++c2) {
+                        const double ar = s_T[2 * (2 * c2 + c)], ai = s_T[2 * (2 * c2 + c) + 1];
+                        const int e = 2 * (4 * (2 * c + x) + 2 * c2 + y);
+                        const double br = s_rho[e], bi = s_rho[e + 1];
+                        sr += ar * br - ai * bi;
+                        si += ar * bi + ai * br;
+                    }
+                __syncwarp();
+                if (lane < 4) s_one[2 * lane] = sr, s_one[2 * lane + 1] = si;
+                __syncwarp();
+                id1 = window_pick<2>(s_one, p.K[1], p.G[1], p.A[1], *p.u[1], p.nK[1], s_T, s_prob, s_M[1], p.chosen[1],
+                                     p.status, report);
+            }
+            if (lane < 16) {
+                s_m[0][lane].x = R(s_M[0][2 * lane]);
+                s_m[0][lane].y = R(s_M[0][2 * lane + 1]);
+                s_m[1][lane].x = R(s_M[1][2 * lane]);
+                s_m[1][lane].y = R(s_M[1][2 * lane + 1]);
+            }
+            if (lane == 0) s_identity[0] = id0, s_identity[1] = id1;
+        }
+        __syncthreads();
+    }
+    const bool ap0 = p.na > 0 && !s_identity[0], ap1 = p.na > 0 && p.nch == 2 && !s_identity[1];
+    const bool wide = p.na == 2 && p.nch == 1;
+
+    // sums of the next window's matrix, as in k_rdm
+    constexpr int NE = 10;
+    R ar[NE], ai[NE], cr[NE], ci[NE];
+#pragma unroll
+    for (int e = 0; e < NE; ++e) ar[e] = ai[e] = cr[e] = ci[e] = 0;
+    auto add = [](R &sum, R &comp, R x) {
+        if constexpr (sizeof(R) == 4) {
+            const R y = x - comp;
+            const R t = sum + y;
+            comp = (t - sum) - y;
+            sum = t;
+        } else {
+            sum += x;
+        }
+    };
+    while (f < groups) {
+        if (ap0 || ap1) {
+            if (wide) {
+#pragma unroll
+                for (int b = 0; b < 4; ++b) {
+                    T2 o[4];
+#pragma unroll
+                    for (int r = 0; r < 4; ++r) {
+                        o[r].x = o[r].y = 0;
+#pragma unroll
+                        for (int c = 0; c < 4; ++c) cmac(o[r], s_m[0][4 * r + c], v[4 * c + b]);
+                    }
+#pragma unroll
+                    for (int r = 0; r < 4; ++r) v[4 * r + b] = o[r];
+                }
+            } else {
+                if (ap0) {
+                    const T2 m00 = s_m[0][0], m01 = s_m[0][1], m10 = s_m[0][2], m11 = s_m[0][3];
+#pragma unroll
+                    for (int i = 0; i < 8; ++i) {
+                        T2 o0, o1;
+                        o0.x = o0.y = o1.x = o1.y = 0;
+                        cmac(o0, m00, v[i]);
+                        cmac(o0, m01, v[i + 8]);
+                        cmac(o1, m10, v[i]);
+                        cmac(o1, m11, v[i + 8]);
+                        v[i] = o0;
+                        v[i + 8] = o1;
+                    }
+                }
+                if (ap1) {
+                    const T2 m00 = s_m[1][0], m01 = s_m[1][1], m10 = s_m[1][2], m11 = s_m[1][3];
+#pragma unroll
+                    for (int i = 0; i < 8; ++i) {
+                        const int j = (i & 3) | ((i & 4) << 1);
+                        T2 o0, o1;
+                        o0.x = o0.y = o1.x = o1.y = 0;
+                        cmac(o0, m00, v[j]);
+                        cmac(o0, m01, v[j + 4]);
+                        cmac(o1, m10, v[j]);
+                        cmac(o1, m11, v[j + 4]);
+                        v[j] = o0;
+                        v[j + 4] = o1;
+                    }
+                }
+            }
+#pragma unroll
+            for (int i = 0; i < 16; ++i) base[p.off[i]] = v[i];
+        }
+        if (p.nb == 2) {
+            int e = 0;
+#pragma unroll
+            for (int b = 0; b < 4; ++b)
+#pragma unroll
+                for (int b2 = b; b2 < 4; ++b2, ++e) {
+                    R sr = 0, si = 0;
+#pragma unroll
+                    for (int a = 0; a < 4; ++a) {
+                        const T2 s = v[4 * a + b], t = v[4 * a + b2];
+                        sr += s.x * t.x + s.y * t.y;
+                        if (b != b2) si += s.y * t.x - s.x * t.y;
+                    }
+                    add(ar[e], cr[e], sr);
+                    if (b != b2) add(ai[e], ci[e], si);
+                }
+        } else if (p.nb == 1) {
+            int e = 0;
+#pragma unroll
+            for (int b = 0; b < 2; ++b)
+#pragma unroll
+                for (int b2 = b; b2 < 2; ++b2, ++e) {
+                    R sr = 0, si = 0;
+#pragma unroll
+                    for (int a = 0; a < 8; ++a) {  // a: this window's qubits and the replaced one
+                        const T2 s = v[4 * (a >> 1) + 2 * b + (a & 1)], t = v[4 * (a >> 1) + 2 * b2 + (a & 1)];
+                        sr += s.x * t.x + s.y * t.y;
+                        if (b != b2) si += s.y * t.x - s.x * t.y;
+                    }
+                    add(ar[e], cr[e], sr);
+                    if (b != b2) add(ai[e], ci[e], si);
+                }
+        }
+        f += stride;
+        if (f < groups) {
+            base = psi + spread(f);
+#pragma unroll
+            for (int i = 0; i < 16; ++i) v[i] = base[p.off[i]];
+        }
+    }
+    if (p.nb == 0) return;
+    // per warp by shuffles, then across the warps in a fixed order
+    __syncthreads();
+    const int width = p.nb == 1 ? 6 : kWindowRow;
+#pragma unroll
+    for (int e = 0; e < NE; ++e) {
+        if (2 * e >= width) break;
+        double sr = double(ar[e]) - double(cr[e]), si = double(ai[e]) - double(ci[e]);
+        for (int o = 16; o > 0; o >>= 1) {
+            sr += __shfl_down_sync(0xffffffffu, sr, o);
+            si += __shfl_down_sync(0xffffffffu, si, o);
+        }
+        if (lane == 0) {
+            s_part[warp][2 * e] = sr;
+            s_part[warp][2 * e + 1] = si;
+        }
+    }
+    __syncthreads();
+    if (int(threadIdx.x) < width) {
+        double t = 0;
+        for (int w = 0; w < kWindowThreads / 32; ++w) t += s_part[w][threadIdx.x];
+        p.out[int64_t(blockIdx.x) * kWindowRow + threadIdx.x] = t;
+    }
+}
+
+template <typename R> static int window_grid(int n)
+{
+    const int64_t groups = int64_t(1) << (n - 4);
+    return grid_for((const void *)k_window<R>, kWindowThreads, 0, (groups + kWindowThreads - 1) / kWindowThreads);
+}
+
+// the bits a window kernel works on: this window's qubits a, the next one's b, others in the place of missing ones
+static void window_bits(WindowParam &p, int n, int na, const int *qa, int nb, const int *qb)
+{
+    int bit[4];
+    uint64_t used = 0;
+    for (int j = 0; j < na; ++j) used |= uint64_t(1) << (bit[j] = n - 1 - qa[j]);
+    for (int j = 0; j < nb; ++j) used |= uint64_t(1) << (bit[2 + j] = n - 1 - qb[j]);
+    int top = n - 1;
+    auto other = [&]() {  // a high bit: neighbouring threads keep neighbouring amplitudes
+        while ((used >> top) & 1) --top;
+        used |= uint64_t(1) << top;
+        return top;
+    };
+    for (int j = na; j < 2; ++j) bit[j] = other();
+    for (int j = nb; j < 2; ++j) bit[2 + j] = other();
+    for (int i = 0; i < 16; ++i) {
+        p.off[i] = 0;
+        for (int j = 0; j < 4; ++j)
+            if ((i >> (3 - j)) & 1) p.off[i] += int64_t(1) << bit[j];
+    }
+    std::copy(bit, bit + 4, p.fixed);
+    std::sort(p.fixed, p.fixed + 4);
+    p.free_bits = n - 4;
+    p.na = na;
+    p.nb = nb;
+}
+
+template <typename R> static hq_status launch_window(const WindowParam &p, void *state, int n, cudaStream_t s)
+{
+    k_window<R><<<window_grid<R>(n), kWindowThreads, 0, s>>>(p, (typename C2<R>::type *)state);
+    return cuda_status("k_window", cudaGetLastError());
+}
+
 // K^dag K as a row-major D x D complex matrix
 static void gram(int D, const double *K, double *G)
 {
@@ -568,10 +970,14 @@ hq_status run_trajectory(void *state, int n, hq_dtype dt, const hq_noisy_op *ops
     // operator, chosen indices, status
     const size_t uoff = hostbuf.size();
     for (const Dev &d : dev) hostbuf.push_back(u[d.ch]);
-    const int width = 2 * rdm_entries<2>();
-    const int grid = std::max(dt == HQ_C64 ? std::max(rdm_grid<float, 1>(n), rdm_grid<float, 2>(n))
+    // (n < 4: the per-channel kernels; a window kernel's threads hold four qubits)
+    const bool windows = n >= 4;
+    const int width = windows ? kWindowRow : 2 * rdm_entries<2>();
+    const int grid = windows ? (dt == HQ_C64 ? window_grid<float>(n) : window_grid<double>(n))
+                   : std::max(dt == HQ_C64 ? std::max(rdm_grid<float, 1>(n), rdm_grid<float, 2>(n))
                                            : std::max(rdm_grid<double, 1>(n), rdm_grid<double, 2>(n)), 1);
-    const size_t nd = hostbuf.size() + size_t(grid) * width + 2 * 16 + 1;
+    // two sets of partial sums: a window kernel writes the next one's while other CTAs still read its own
+    const size_t nd = hostbuf.size() + size_t(2) * grid * width + 2 * 16 + 1;
     const size_t bytes = nd * sizeof(double) + sizeof(int) * (dev.size() + 1);
     char *ws = nullptr;
     if (!dev.empty()) {
@@ -586,7 +992,7 @@ hq_status run_trajectory(void *state, int n, hq_dtype dt, const hq_noisy_op *ops
     }
     double *dbuf = reinterpret_cast<double *>(ws);
     double *partials = dbuf ? dbuf + hostbuf.size() : nullptr;
-    double *sel = partials ? partials + size_t(grid) * width : nullptr;
+    double *sel = partials ? partials + size_t(2) * grid * width : nullptr;
     int *chosen_dev = ws ? reinterpret_cast<int *>(ws + nd * sizeof(double)) : nullptr;
     int *status_dev = chosen_dev ? chosen_dev + dev.size() : nullptr;
 
@@ -599,6 +1005,27 @@ hq_status run_trajectory(void *state, int n, hq_dtype dt, const hq_noisy_op *ops
         run.clear();
         return r;
     };
+    // windows of device-sampled channels (k_window)
+    size_t done = 0;      // channels before this one are in launched windows
+    bool fed = false;     // the partial sums of the next window are there
+    int side = 0;         // the set that holds them
+    auto applied_between = [&](int x) {  // an operator applied between channels x and x + 1
+        for (int j = dev[x].op + 1; j < dev[x + 1].op; ++j)
+            if (plan[j] == 0 || plan[j] == 1) return true;
+        return false;
+    };
+    auto shares_qubit = [&](int x, int y) {
+        const hq_noisy_op &a = ops[dev[x].op], &b = ops[dev[y].op];
+        for (int i = 0; i < a.k; ++i)
+            for (int j = 0; j < b.k; ++j)
+                if (a.qubits[i] == b.qubits[j]) return true;
+        return false;
+    };
+    auto window_end = [&](size_t x) {  // last channel of the window that starts with channel x
+        const bool two = x + 1 < dev.size() && ops[dev[x].op].k == 1 && ops[dev[x + 1].op].k == 1 &&
+                         !shares_qubit(int(x), int(x) + 1) && !applied_between(int(x));
+        return int(x) + (two ? 1 : 0);
+    };
     for (int i = 0; i < nops && st == HQ_OK; ++i) {
         if (plan[i] == 0 || plan[i] == 1) {
             hq_gate g;
@@ -609,6 +1036,61 @@ hq_status run_trajectory(void *state, int n, hq_dtype dt, const hq_noisy_op *ops
             run.push_back(g);
         }
         if (plan[i] != 3) continue;
+        if (windows) {
+            if (di < done) {  // the second channel of the window before
+                ++di;
+                continue;
+            }
+            if ((st = flush()) != HQ_OK) break;
+            const int last = window_end(di);
+            // the next window's sums ride along when nothing is applied between and the qubits differ
+            int next_end = -1;
+            if (last + 1 < int(dev.size()) && !applied_between(last)) {
+                next_end = window_end(last + 1);
+                for (int x = int(di); x <= last; ++x)
+                    for (int y = last + 1; y <= next_end; ++y)
+                        if (shares_qubit(x, y)) next_end = -1;
+            }
+            auto qubits_of = [&](int first, int end, int *q) {
+                int k = 0;
+                for (int x = first; x <= end; ++x)
+                    for (int j = 0; j < ops[dev[x].op].k; ++j) q[k++] = ops[dev[x].op].qubits[j];
+                return k;
+            };
+            int qa[2], qb[2];
+            const int na = qubits_of(int(di), last, qa);
+            WindowParam w;
+            if (!fed) {
+                std::memset(&w, 0, sizeof(w));
+                window_bits(w, n, 0, nullptr, na, qa);
+                w.out = partials + size_t(side) * grid * width;
+                st = dt == HQ_C64 ? launch_window<float>(w, state, n, s) : launch_window<double>(w, state, n, s);
+                if (st != HQ_OK) break;
+            }
+            std::memset(&w, 0, sizeof(w));
+            const int nb = next_end < 0 ? 0 : qubits_of(last + 1, next_end, qb);
+            window_bits(w, n, na, qa, nb, qb);
+            w.nch = last - int(di) + 1;
+            for (int x = 0; x < w.nch; ++x) {
+                const Dev &d = dev[di + x];
+                w.K[x] = dbuf + d.koff;
+                w.G[x] = dbuf + d.goff;
+                w.A[x] = dbuf + d.aoff;
+                w.u[x] = dbuf + uoff + di + x;
+                w.nK[x] = ops[d.op].nkraus;
+                w.chosen[x] = chosen_dev + di + x;
+            }
+            w.status = status_dev;
+            w.in = partials + size_t(side) * grid * width;
+            w.rows = grid;
+            side ^= 1;
+            w.out = partials + size_t(side) * grid * width;
+            st = dt == HQ_C64 ? launch_window<float>(w, state, n, s) : launch_window<double>(w, state, n, s);
+            fed = nb > 0;
+            done = size_t(last) + 1;
+            ++di;
+            continue;
+        }
         if ((st = flush()) != HQ_OK) break;
         const Dev &d = dev[di];
         PickArgs a;

@@ -166,3 +166,46 @@ def test_trajectory_folds_gates_into_two_qubit_channels(hq, dtype):
         assert got.tolist() == want, trial
         err = np.abs(st.cpu().numpy().astype(np.complex128) - psi).max()
         assert err <= (1e-12 if dtype == "complex128" else 2e-6), (trial, err)
+
+
+@pytest.mark.parametrize("dtype", ["complex64", "complex128"])
+@pytest.mark.parametrize("n", [2, 3, 4, 5, 7, 10])
+def test_chains_of_state_dependent_channels(hq, n, dtype):
+    """Runs of channels that share a pass over the state two at a time: on
+    distinct qubits in every order (lowest and highest bits), the same qubit
+    twice, two-qubit channels between one-qubit ones, an applied gate in
+    between: branches and states against the oracle."""
+    rng = np.random.default_rng(40 + n)  # input only
+    sm = C.SplitMix64(n)
+    ops = []
+    for block in range(6):
+        order = [int(q) for q in rng.permutation(n)]
+        if block == 2:
+            order = order[:1] * 3 + order
+        for q in order:
+            if rng.random() < 0.6:
+                ops.append(("gate", (q,), C.random_unitary(1, sm)))
+            ops.append(("kraus", (q,), C.amplitude_damping(0.4, 0.2) if rng.random() < 0.7 else random_kraus(1, 3, rng)))
+            if rng.random() < 0.2:
+                pair = tuple(int(x) for x in rng.choice(n, 2, replace=False))
+                ops.append(("kraus", pair, random_kraus(2, 3, rng)))
+            if rng.random() < 0.15:
+                pair = tuple(int(x) for x in rng.choice(n, 2, replace=False))
+                ops.append(("gate", pair, C.cz()))
+    u = rng.random(sum(1 for o in ops if o[0] == "kraus"))
+    tokens = "".join("01+-"[int(x)] for x in rng.integers(0, 4, n))
+    psi, want, c = oracle.state_init(n, tokens), [], 0
+    for kind, qs, m in ops:
+        if kind == "gate":
+            psi = oracle.apply_gate(psi, n, qs, m)
+        else:
+            i, psi = N.trajectory_step(psi, n, list(qs), m, u[c])
+            want.append(i)
+            c += 1
+    st = torch.empty(1 << n, dtype=getattr(torch, dtype), device="cuda")
+    hq.hq_state_init(st, tokens)
+    got = hq.hq_run_trajectory(st, ops, u)
+    assert got.tolist() == want
+    # complex64: some 100 operators, each rounding the state by a few 2^-24
+    err = np.linalg.norm(st.cpu().numpy().astype(np.complex128) - psi)
+    assert err <= (1e-12 if dtype == "complex128" else 2e-5)
