@@ -18,6 +18,7 @@
 #include <cstring>
 #include <vector>
 
+#include "hq_cp_async.cuh"
 #include "hq_fault.cuh"
 #include "hq_internal.cuh"
 
@@ -444,7 +445,7 @@ static hq_status sample_on_device(void *state, int n, const int *qubits, PickArg
 // Bound: HBM (two channels at n = 24: 268 MB, 40 us at the copy bandwidth), with
 // about 5 us of FP64 latency per launch for the pick; complex128 the FP64 pipe.
 // ----------------------------------------------------------------------------
-constexpr int kWindowRow = 20;  // doubles per CTA: 10 complex entries of the upper triangle
+constexpr int kWindowRow = 20;  // sums per CTA: 10 complex entries of the upper triangle
 struct WindowParam {
     int64_t off[16];   // flat offset of local index 4 a + b (a: this window's qubits, b: the next one's; first qubit
                        // most significant)
@@ -456,9 +457,9 @@ struct WindowParam {
     int nK[2];
     int *chosen[2];
     int *status;
-    const double *in;  // partial sums for this window: `rows` rows of kWindowRow
+    const void *in;    // partial sums for this window: `rows` rows of kWindowRow Pair<R>
     int rows;
-    double *out;       // partial sums for the next window, one row per CTA
+    void *out;         // partial sums for the next window, one row per CTA
 };
 
 // One warp: the branch of a channel on D levels with reduced density matrix
@@ -523,7 +524,7 @@ __device__ __forceinline__ bool window_pick(const double *rho0, const double *K,
     if (!(total > 0)) pick = -1;
     double mr = x == y ? 1.0 : 0.0, mi = 0;
     if (pick >= 0) {
-        const double sc = 1.0 / sqrt(ppick);
+        const double sc = rsqrt(ppick);
         const double *Kp = K + size_t(pick) * 2 * DD;
         mr = 0;
 #pragma unroll
@@ -548,16 +549,91 @@ __device__ __forceinline__ bool window_pick(const double *rho0, const double *K,
     return identity;
 }
 
-constexpr int kWindowThreads = 256;
+// Sums of a window kernel: pairs (high, low) of the state's real type, joined by error-free additions (Knuth's
+// two-sum; the pair carries 48 bits for FP32).  An FP64 instruction takes a GB300 SM's quarter 64 cycles whatever its
+// lanes do: joined as doubles, the 20 sums of each of the 16 warps were 21 of a launch's 83 us.
+template <typename R> struct Pair {
+    R h, l;
+};
+__device__ __forceinline__ Pair<float> pair_add(Pair<float> a, Pair<float> b)
+{
+    const float t = a.h + b.h, z = t - a.h;
+    const float e = ((a.h - (t - z)) + (b.h - z)) + (a.l + b.l);
+    Pair<float> r;
+    r.h = t + e;
+    r.l = e - (r.h - t);
+    return r;
+}
+__device__ __forceinline__ Pair<double> pair_add(Pair<double> a, Pair<double> b) { return {a.h + b.h, 0.0}; }
+// a thread's compensated sum
+__device__ __forceinline__ Pair<float> pair_of(float sum, float comp)
+{
+    const float h = sum - comp;
+    return {h, (sum - h) - comp};
+}
+__device__ __forceinline__ Pair<double> pair_of(double sum, double) { return {sum, 0.0}; }
+// lane 0: the sum over the warp
+template <typename R> __device__ __forceinline__ Pair<R> warp_join(Pair<R> v)
+{
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        Pair<R> w;
+        w.h = __shfl_down_sync(0xffffffffu, v.h, o);
+        w.l = sizeof(R) == 4 ? __shfl_down_sync(0xffffffffu, v.l, o) : R(0);
+        v = pair_add(v, w);
+    }
+    return v;
+}
+
+// (v0, v1) <- m (v0, v1), m row-major 2 x 2; complex64 with packed FMAs in cmac's order
+__device__ __forceinline__ float2 swap_halves(float2 v) { return make_float2(v.y, v.x); }
+__device__ __forceinline__ double2 swap_halves(double2 v) { return make_double2(v.y, v.x); }
+__device__ __forceinline__ void apply_pair(const float2 *m, float2 &v0, float2 &v1)
+{
+    const float2 w0 = swap_halves(v0), w1 = swap_halves(v1);
+    auto row = [&](const float2 a, const float2 b) {
+        float2 o = pk_mul(make_float2(a.x, a.x), v0);
+        o = pk_fma(make_float2(-a.y, a.y), w0, o);
+        o = pk_fma(make_float2(b.x, b.x), v1, o);
+        return pk_fma(make_float2(-b.y, b.y), w1, o);
+    };
+    const float2 o0 = row(m[0], m[1]), o1 = row(m[2], m[3]);
+    v0 = o0;
+    v1 = o1;
+}
+__device__ __forceinline__ void apply_pair(const double2 *m, double2 &v0, double2 &v1)
+{
+    double2 o0, o1;
+    o0.x = o0.y = o1.x = o1.y = 0;
+    cmac(o0, m[0], v0);
+    cmac(o0, m[1], v1);
+    cmac(o1, m[2], v0);
+    cmac(o1, m[3], v1);
+    v0 = o0;
+    v1 = o1;
+}
+// acc += (a.x b.x, a.y b.y)
+__device__ __forceinline__ void mac2(float2 &acc, float2 a, float2 b) { acc = pk_fma(a, b, acc); }
+__device__ __forceinline__ void mac2(double2 &acc, double2 a, double2 b)
+{
+    acc.x = fma(a.x, b.x, acc.x);
+    acc.y = fma(a.y, b.y, acc.y);
+}
+
+constexpr int kWindowOps = 64;  // doubles of K (and of G) that are staged in shared memory
+
+// one CTA per SM: few partial sums to read back (152 rows instead of 304: the pick's FP64 additions halve twice over)
+constexpr int kWindowThreads = 512;
 
 template <typename R>
-__global__ void __launch_bounds__(kWindowThreads, sizeof(R) == 4 ? 2 : 1) k_window(const __grid_constant__ WindowParam p,
+__global__ void __launch_bounds__(kWindowThreads, 1) k_window(const __grid_constant__ WindowParam p,
                                                               typename C2<R>::type *__restrict__ psi)
 {
     using T2 = typename C2<R>::type;
-    __shared__ double s_part[kWindowThreads / 32][kWindowRow];
+    __shared__ Pair<R> s_part[kWindowThreads / 32][kWindowRow];
     __shared__ double s_rho[32], s_one[32], s_T[32], s_prob[kMaxKraus], s_M[2][32];
     __shared__ T2 s_m[2][16];
+    __shared__ double s_op[2][3][kWindowOps], s_u[2];  // K, G, A of each channel
     __shared__ int s_identity[2];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int64_t groups = int64_t(1) << p.free_bits, stride = int64_t(gridDim.x) * blockDim.x;
@@ -570,26 +646,53 @@ __global__ void __launch_bounds__(kWindowThreads, sizeof(R) == 4 ? 2 : 1) k_wind
         }
         return x;
     };
+    // complex64: a thread's groups come through its own slots of shared memory (cp.async; nobody else reads them, so
+    // no barrier), two groups in flight: the first two under the pick, the later ones under the groups before them.
+    // Three stages: a stage is filled again only after the arithmetic on what was read from it.
+    constexpr bool kStaged = sizeof(R) == 4;
+    extern __shared__ __align__(16) unsigned char s_stage[];
+    T2 *const slot = reinterpret_cast<T2 *>(s_stage) + threadIdx.x;  // [stage][16][kWindowThreads]
     T2 v[16];
     int64_t f = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
-    // the first group's loads run under the pick
-    T2 *base = psi + (f < groups ? spread(f) : 0);
-    if (f < groups) {
+    int stage = 0;
+    auto fetch = [&](int64_t g, int to) {
+        if (g < groups) {
+            const T2 *const from = psi + spread(g);
 #pragma unroll
-        for (int i = 0; i < 16; ++i) v[i] = base[p.off[i]];
+            for (int i = 0; i < 16; ++i) cp_async8(slot + (16 * to + i) * kWindowThreads, from + p.off[i]);
+        }
+        cp_async_commit();
+    };
+    if constexpr (kStaged) {
+        fetch(f, 0);
+        fetch(f + stride, 1);
+    }
+    // small operators staged by the CTA while its first warps read the sums
+    for (int x = 0; x < p.nch; ++x) {
+        const int DD = p.nch == 2 || p.na == 1 ? 4 : 16, n2 = p.nK[x] * 2 * DD;
+        if (n2 <= kWindowOps)
+            for (int i = threadIdx.x; i < n2; i += blockDim.x) {
+                s_op[x][0][i] = p.K[x][i];
+                s_op[x][1][i] = p.G[x][i];
+            }
+        if (int(threadIdx.x) < 2 * DD) s_op[x][2][threadIdx.x] = p.A[x][threadIdx.x];
+        if (threadIdx.x == 0) s_u[x] = *p.u[x];
     }
     if (p.na > 0) {
         // the CTAs' sums, in a fixed order: rows warp by warp, one column per lane
         const int width = p.na == 1 ? 6 : kWindowRow;
-        double t = 0;
+        const Pair<R> *const in = reinterpret_cast<const Pair<R> *>(p.in);
+        Pair<R> part = {R(0), R(0)};
         if (lane < width)
-            for (int r = warp; r < p.rows; r += kWindowThreads / 32) t += p.in[int64_t(r) * kWindowRow + lane];
-        if (lane < kWindowRow) s_part[warp][lane] = t;
+            for (int r = warp; r < p.rows; r += kWindowThreads / 32)
+                part = pair_add(part, in[int64_t(r) * kWindowRow + lane]);
+        if (lane < kWindowRow) s_part[warp][lane] = part;
         __syncthreads();
         if (warp == 0) {
-            t = 0;
+            part = {R(0), R(0)};
             if (lane < width)
-                for (int w = 0; w < kWindowThreads / 32; ++w) t += s_part[w][lane];
+                for (int w = 0; w < kWindowThreads / 32; ++w) part = pair_add(part, s_part[w][lane]);
+            const double t = double(part.h) + double(part.l);
             // upper triangle -> full matrix
             const int D = 1 << p.na;
             if (lane < width) {
@@ -602,10 +705,17 @@ __global__ void __launch_bounds__(kWindowThreads, sizeof(R) == 4 ? 2 : 1) k_wind
             __syncwarp();
             bool id0, id1 = true;
             const bool report = blockIdx.x == 0;
+            const int DD = p.nch == 2 || p.na == 1 ? 4 : 16;
+            const double *K[2], *G[2];
+            for (int x = 0; x < 2; ++x) {
+                const bool staged = p.nK[x] * 2 * DD <= kWindowOps;
+                K[x] = staged ? s_op[x][0] : p.K[x];
+                G[x] = staged ? s_op[x][1] : p.G[x];
+            }
             if (p.nch == 1) {
-                id0 = p.na == 1 ? window_pick<2>(s_rho, p.K[0], p.G[0], p.A[0], *p.u[0], p.nK[0], s_T, s_prob, s_M[0],
+                id0 = p.na == 1 ? window_pick<2>(s_rho, K[0], G[0], s_op[0][2], s_u[0], p.nK[0], s_T, s_prob, s_M[0],
                                                  p.chosen[0], p.status, report)
-                                : window_pick<4>(s_rho, p.K[0], p.G[0], p.A[0], *p.u[0], p.nK[0], s_T, s_prob, s_M[0],
+                                : window_pick<4>(s_rho, K[0], G[0], s_op[0][2], s_u[0], p.nK[0], s_T, s_prob, s_M[0],
                                                  p.chosen[0], p.status, report);
             } else {
                 // the first qubit's partial trace
@@ -615,7 +725,7 @@ __global__ void __launch_bounds__(kWindowThreads, sizeof(R) == 4 ? 2 : 1) k_wind
                         s_rho[2 * (4 * (2 * a) + 2 * a2) + im] + s_rho[2 * (4 * (2 * a + 1) + 2 * a2 + 1) + im];
                 }
                 __syncwarp();
-                id0 = window_pick<2>(s_one, p.K[0], p.G[0], p.A[0], *p.u[0], p.nK[0], s_T, s_prob, s_M[0], p.chosen[0],
+                id0 = window_pick<2>(s_one, K[0], G[0], s_op[0][2], s_u[0], p.nK[0], s_T, s_prob, s_M[0], p.chosen[0],
                                      p.status, report);
                 // Q = M^dag M, then the second qubit's matrix after the first operator
                 const int x = (lane >> 1) & 1, y = lane & 1;
@@ -644,7 +754,7 @@ __global__ void __launch_bounds__(kWindowThreads, sizeof(R) == 4 ? 2 : 1) k_wind
                 __syncwarp();
                 if (lane < 4) s_one[2 * lane] = sr, s_one[2 * lane + 1] = si;
                 __syncwarp();
-                id1 = window_pick<2>(s_one, p.K[1], p.G[1], p.A[1], *p.u[1], p.nK[1], s_T, s_prob, s_M[1], p.chosen[1],
+                id1 = window_pick<2>(s_one, K[1], G[1], s_op[1][2], s_u[1], p.nK[1], s_T, s_prob, s_M[1], p.chosen[1],
                                      p.status, report);
             }
             if (lane < 16) {
@@ -676,6 +786,17 @@ __global__ void __launch_bounds__(kWindowThreads, sizeof(R) == 4 ? 2 : 1) k_wind
         }
     };
     while (f < groups) {
+        T2 *const base = psi + spread(f);
+        if constexpr (kStaged) {
+            cp_async_wait<1>();
+#pragma unroll
+            for (int i = 0; i < 16; ++i) v[i] = slot[(16 * stage + i) * kWindowThreads];
+            fetch(f + 2 * stride, stage == 0 ? 2 : stage - 1);
+            stage = stage == 2 ? 0 : stage + 1;
+        } else {
+#pragma unroll
+            for (int i = 0; i < 16; ++i) v[i] = base[p.off[i]];
+        }
         if (ap0 || ap1) {
             if (wide) {
 #pragma unroll
@@ -692,32 +813,14 @@ __global__ void __launch_bounds__(kWindowThreads, sizeof(R) == 4 ? 2 : 1) k_wind
                 }
             } else {
                 if (ap0) {
-                    const T2 m00 = s_m[0][0], m01 = s_m[0][1], m10 = s_m[0][2], m11 = s_m[0][3];
 #pragma unroll
-                    for (int i = 0; i < 8; ++i) {
-                        T2 o0, o1;
-                        o0.x = o0.y = o1.x = o1.y = 0;
-                        cmac(o0, m00, v[i]);
-                        cmac(o0, m01, v[i + 8]);
-                        cmac(o1, m10, v[i]);
-                        cmac(o1, m11, v[i + 8]);
-                        v[i] = o0;
-                        v[i + 8] = o1;
-                    }
+                    for (int i = 0; i < 8; ++i) apply_pair(s_m[0], v[i], v[i + 8]);
                 }
                 if (ap1) {
-                    const T2 m00 = s_m[1][0], m01 = s_m[1][1], m10 = s_m[1][2], m11 = s_m[1][3];
 #pragma unroll
                     for (int i = 0; i < 8; ++i) {
                         const int j = (i & 3) | ((i & 4) << 1);
-                        T2 o0, o1;
-                        o0.x = o0.y = o1.x = o1.y = 0;
-                        cmac(o0, m00, v[j]);
-                        cmac(o0, m01, v[j + 4]);
-                        cmac(o1, m10, v[j]);
-                        cmac(o1, m11, v[j + 4]);
-                        v[j] = o0;
-                        v[j + 4] = o1;
+                        apply_pair(s_m[1], v[j], v[j + 4]);
                     }
                 }
             }
@@ -730,15 +833,16 @@ __global__ void __launch_bounds__(kWindowThreads, sizeof(R) == 4 ? 2 : 1) k_wind
             for (int b = 0; b < 4; ++b)
 #pragma unroll
                 for (int b2 = b; b2 < 4; ++b2, ++e) {
-                    R sr = 0, si = 0;
+                    T2 re, im;
+                    re.x = re.y = im.x = im.y = 0;
 #pragma unroll
                     for (int a = 0; a < 4; ++a) {
                         const T2 s = v[4 * a + b], t = v[4 * a + b2];
-                        sr += s.x * t.x + s.y * t.y;
-                        if (b != b2) si += s.y * t.x - s.x * t.y;
+                        mac2(re, s, t);
+                        if (b != b2) mac2(im, swap_halves(s), t);
                     }
-                    add(ar[e], cr[e], sr);
-                    if (b != b2) add(ai[e], ci[e], si);
+                    add(ar[e], cr[e], re.x + re.y);
+                    if (b != b2) add(ai[e], ci[e], im.x - im.y);
                 }
         } else if (p.nb == 1) {
             int e = 0;
@@ -746,53 +850,46 @@ __global__ void __launch_bounds__(kWindowThreads, sizeof(R) == 4 ? 2 : 1) k_wind
             for (int b = 0; b < 2; ++b)
 #pragma unroll
                 for (int b2 = b; b2 < 2; ++b2, ++e) {
-                    R sr = 0, si = 0;
+                    T2 re, im;
+                    re.x = re.y = im.x = im.y = 0;
 #pragma unroll
                     for (int a = 0; a < 8; ++a) {  // a: this window's qubits and the replaced one
                         const T2 s = v[4 * (a >> 1) + 2 * b + (a & 1)], t = v[4 * (a >> 1) + 2 * b2 + (a & 1)];
-                        sr += s.x * t.x + s.y * t.y;
-                        if (b != b2) si += s.y * t.x - s.x * t.y;
+                        mac2(re, s, t);
+                        if (b != b2) mac2(im, swap_halves(s), t);
                     }
-                    add(ar[e], cr[e], sr);
-                    if (b != b2) add(ai[e], ci[e], si);
+                    add(ar[e], cr[e], re.x + re.y);
+                    if (b != b2) add(ai[e], ci[e], im.x - im.y);
                 }
         }
         f += stride;
-        if (f < groups) {
-            base = psi + spread(f);
-#pragma unroll
-            for (int i = 0; i < 16; ++i) v[i] = base[p.off[i]];
-        }
     }
+    if constexpr (kStaged) cp_async_wait<0>();
     if (p.nb == 0) return;
-    // per warp by shuffles, then across the warps in a fixed order
+    // every thread's sums to shared memory; lane by lane over the warps, then each sum's 32 lanes by shuffles (fixed
+    // order; five shuffle levels of all 20 sums in every warp took 3 us)
     __syncthreads();
+    Pair<R> *const all = reinterpret_cast<Pair<R> *>(s_stage);  // [warp][sum][lane]
     const int width = p.nb == 1 ? 6 : kWindowRow;
 #pragma unroll
-    for (int e = 0; e < NE; ++e) {
-        if (2 * e >= width) break;
-        double sr = double(ar[e]) - double(cr[e]), si = double(ai[e]) - double(ci[e]);
-        for (int o = 16; o > 0; o >>= 1) {
-            sr += __shfl_down_sync(0xffffffffu, sr, o);
-            si += __shfl_down_sync(0xffffffffu, si, o);
+    for (int e = 0; e < NE; ++e)
+        if (2 * e < width) {
+            all[(warp * kWindowRow + 2 * e) * 32 + lane] = pair_of(ar[e], cr[e]);
+            all[(warp * kWindowRow + 2 * e + 1) * 32 + lane] = pair_of(ai[e], ci[e]);
         }
-        if (lane == 0) {
-            s_part[warp][2 * e] = sr;
-            s_part[warp][2 * e + 1] = si;
-        }
-    }
     __syncthreads();
-    if (int(threadIdx.x) < width) {
-        double t = 0;
-        for (int w = 0; w < kWindowThreads / 32; ++w) t += s_part[w][threadIdx.x];
-        p.out[int64_t(blockIdx.x) * kWindowRow + threadIdx.x] = t;
+    for (int j = warp; j < width; j += kWindowThreads / 32) {
+        Pair<R> t = all[j * 32 + lane];
+        for (int w = 1; w < kWindowThreads / 32; ++w) t = pair_add(t, all[(w * kWindowRow + j) * 32 + lane]);
+        t = warp_join(t);
+        if (lane == 0) reinterpret_cast<Pair<R> *>(p.out)[int64_t(blockIdx.x) * kWindowRow + j] = t;
     }
 }
 
 template <typename R> static int window_grid(int n)
 {
     const int64_t groups = int64_t(1) << (n - 4);
-    return grid_for((const void *)k_window<R>, kWindowThreads, 0, (groups + kWindowThreads - 1) / kWindowThreads);
+    return int(std::min<int64_t>(sm_count(), (groups + kWindowThreads - 1) / kWindowThreads));
 }
 
 // the bits a window kernel works on: this window's qubits a, the next one's b, others in the place of missing ones
@@ -824,7 +921,11 @@ static void window_bits(WindowParam &p, int n, int na, const int *qa, int nb, co
 
 template <typename R> static hq_status launch_window(const WindowParam &p, void *state, int n, cudaStream_t s)
 {
-    k_window<R><<<window_grid<R>(n), kWindowThreads, 0, s>>>(p, (typename C2<R>::type *)state);
+    // complex64: three stages of groups; then (and in complex128 only) the threads' sums
+    const size_t smem = std::max(sizeof(R) == 4 ? size_t(3) * 16 * kWindowThreads * sizeof(float2) : size_t(0),
+                                 size_t(kWindowThreads) * kWindowRow * sizeof(Pair<R>));
+    occupancy((const void *)k_window<R>, kWindowThreads, smem);  // (sets the kernel's shared-memory limit)
+    k_window<R><<<window_grid<R>(n), kWindowThreads, smem, s>>>(p, (typename C2<R>::type *)state);
     return cuda_status("k_window", cudaGetLastError());
 }
 
@@ -972,7 +1073,7 @@ hq_status run_trajectory(void *state, int n, hq_dtype dt, const hq_noisy_op *ops
     for (const Dev &d : dev) hostbuf.push_back(u[d.ch]);
     // (n < 4: the per-channel kernels; a window kernel's threads hold four qubits)
     const bool windows = n >= 4;
-    const int width = windows ? kWindowRow : 2 * rdm_entries<2>();
+    const int width = windows ? kWindowRow * (dt == HQ_C64 ? 1 : 2) : 2 * rdm_entries<2>();  // doubles per row
     const int grid = windows ? (dt == HQ_C64 ? window_grid<float>(n) : window_grid<double>(n))
                    : std::max(dt == HQ_C64 ? std::max(rdm_grid<float, 1>(n), rdm_grid<float, 2>(n))
                                            : std::max(rdm_grid<double, 1>(n), rdm_grid<double, 2>(n)), 1);
