@@ -10,6 +10,7 @@ from __future__ import annotations
 
 import ctypes
 import os
+import struct
 from typing import Iterable, Sequence
 
 import numpy as np
@@ -183,6 +184,29 @@ def _stream(stream):
     return ctypes.c_void_p(stream.cuda_stream)
 
 
+def _data_ptr(a: np.ndarray) -> int:
+    return a.__array_interface__["data"][0]
+
+
+# one record of each C struct by its number of qubits (native alignment): a whole struct per call instead of one
+# ctypes attribute per field
+_PACK_GATE = [struct.Struct(f"@i{k}i{4 * (HQ_MAX_K - k)}xP") for k in range(HQ_MAX_K + 1)]
+_PACK_NOISY = [struct.Struct(f"@i{k}i{4 * (HQ_MAX_K - k)}xiP") for k in range(HQ_MAX_K + 1)]
+_GATE_BYTES = ctypes.sizeof(hq_gate)
+_NOISY_BYTES = ctypes.sizeof(hq_noisy_op)
+
+
+def _matrix_ptr(m, known: dict, keep: list) -> int:
+    """Address of the matrix as contiguous complex128; `known`: the addresses of this call's matrices by object
+    (circuits repeat a few gates many times; `keep` holds every object and copy until the call returns)."""
+    p = known.get(id(m))
+    if p is None:
+        c = np.ascontiguousarray(m, np.complex128)
+        keep.append((m, c))
+        p = known[id(m)] = _data_ptr(c)
+    return p
+
+
 def _gate_struct(qubits: Sequence[int], matrix: np.ndarray, keep: list) -> hq_gate:
     m = np.ascontiguousarray(matrix, np.complex128)
     keep.append(m)
@@ -197,9 +221,17 @@ def _gate_struct(qubits: Sequence[int], matrix: np.ndarray, keep: list) -> hq_ga
 def _gates_array(gates: Iterable, keep: list):
     gl = list(gates)
     arr = (hq_gate * max(1, len(gl)))()
+    known: dict = {}
+    at = 0
     for i, g in enumerate(gl):
         qs, m = (g.qubits, g.matrix) if hasattr(g, "qubits") else g
-        arr[i] = _gate_struct(qs, m, keep)
+        p = _matrix_ptr(m, known, keep)
+        k = len(qs)
+        try:
+            _PACK_GATE[k].pack_into(arr, at, k, *qs, p)
+        except (struct.error, IndexError):  # qubits that are not integers but convert to them; too many
+            arr[i] = _gate_struct(qs, m, keep)
+        at += _GATE_BYTES
     return arr, len(gl)
 
 
@@ -404,8 +436,21 @@ def hq_reduced_density_matrix(state, qubits: Sequence[int], stream=None) -> np.n
     return out.view(np.complex128).reshape(1 << k, 1 << k)
 
 
+def _stacked(ops) -> np.ndarray:
+    """The matrices one after another, contiguous complex128."""
+    ops = list(ops)
+    if ops and all(type(m) is np.ndarray for m in ops):
+        shapes = {m.shape for m in ops}
+        if len(shapes) == 1:
+            shape = shapes.pop()
+            if len(shape) == 2:  # one concatenation: a quarter of np.stack's time
+                out = np.concatenate(ops).reshape((len(ops),) + shape)
+                return np.ascontiguousarray(out, np.complex128)
+    return np.ascontiguousarray(np.stack([np.asarray(m, np.complex128) for m in ops]), np.complex128)
+
+
 def _kraus_block(kraus) -> np.ndarray:
-    return np.ascontiguousarray(np.stack([np.asarray(K, np.complex128) for K in kraus]), np.complex128)
+    return _stacked(kraus)
 
 
 def hq_apply_kraus_sampled(state, qubits: Sequence[int], kraus, u: float, stream=None) -> int:
@@ -428,22 +473,28 @@ def hq_run_trajectory(state, ops, u, engine: str | int = "auto", tc_min_k: int =
     ptr, n, dt = _state_args(state)
     keep: list = []
     arr = (hq_noisy_op * max(1, len(ops)))()
+    known: dict = {}
+    nch = 0
     for i, (kind, qubits, m) in enumerate(ops):
-        arr[i].k = len(qubits)
-        for j, q in enumerate(qubits):
-            arr[i].qubits[j] = int(q)
         if kind == "gate":
-            mm = np.ascontiguousarray(m, np.complex128)
-            arr[i].nkraus = 0
+            p, nk = _matrix_ptr(m, known, keep), 0
         elif kind == "kraus":
             mm = _kraus_block(m)
-            arr[i].nkraus = len(mm)
+            keep.append(mm)
+            p, nk = _data_ptr(mm), len(mm)
+            nch += 1
         else:
             raise ValueError(f"unknown op kind {kind!r}")
-        keep.append(mm)
-        arr[i].matrix = mm.ctypes.data
+        k = len(qubits)
+        try:
+            _PACK_NOISY[k].pack_into(arr, i * _NOISY_BYTES, k, *qubits, nk, p)
+        except (struct.error, IndexError):
+            h = arr[i]
+            h.k = k
+            for j, q in enumerate(qubits):
+                h.qubits[j] = int(q)
+            h.nkraus, h.matrix = nk, p
     uu = np.ascontiguousarray(u, np.float64)
-    nch = sum(1 for kind, _, _ in ops if kind == "kraus")
     if uu.size < nch:
         raise ValueError("one uniform per channel is needed")
     chosen = np.full(max(1, nch), -1, np.int32)
@@ -477,16 +528,15 @@ def hq_expectation_static(state, H, stream=None) -> float:
 
 def _ops_array(circuit, keep: list):
     arr = (hq_op * max(1, len(circuit.gates)))()
+    known: dict = {}
     for i, g in enumerate(circuit.gates):
         op = arr[i]
         op.k = g.k
         for j, q in enumerate(g.qubits):
             op.qubits[j] = int(q)
         if g.matrix is not None:
-            m = np.ascontiguousarray(g.matrix, np.complex128)
-            keep.append(m)
             op.kind = HQ_OP_MATRIX
-            op.matrix = m.ctypes.data
+            op.matrix = _matrix_ptr(g.matrix, known, keep)
         else:
             op.kind = HQ_OP_ROT
             op.axis = ord(g.axis)
@@ -610,7 +660,7 @@ def _dm_args(rho):
 
 
 def _ops_block(ops) -> np.ndarray:
-    return np.ascontiguousarray(np.stack([np.asarray(m, np.complex128) for m in ops]), np.complex128)
+    return _stacked(ops)
 
 
 def hq_dm_superop(left, right=None, s=None) -> np.ndarray:
