@@ -28,6 +28,9 @@
  *     exception crosses the boundary.
  *   - Threading: entry points may be called from several host threads; the
  *     per-device library state is set up once under a lock.
+ *   - Device scratch: stream-ordered, from a memory pool that the library keeps
+ *     per device (at most 16 MB stay mapped between calls).  Results of
+ *     synchronous calls come back through a small pinned buffer per host thread.
  */
 #ifndef HQ_H
 #define HQ_H

@@ -146,6 +146,173 @@ cudaEvent_t call_event()
     return ev[dev];
 }
 
+// ----------------------------------------------------------------------------
+// device scratch
+// ----------------------------------------------------------------------------
+namespace {
+constexpr uint64_t kScratchKeep = 16 << 20;  // bytes a device's pool keeps mapped between calls
+
+cudaMemPool_t scratch_pool()
+{
+    static std::mutex mu;
+    static cudaMemPool_t pools[64] = {nullptr};
+    static bool tried[64] = {false};
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return nullptr;
+    std::lock_guard<std::mutex> lk(mu);
+    if (!tried[dev]) {
+        tried[dev] = true;
+        cudaMemPoolProps pr;
+        std::memset(&pr, 0, sizeof(pr));
+        pr.allocType = cudaMemAllocationTypePinned;
+        pr.location.type = cudaMemLocationTypeDevice;
+        pr.location.id = dev;
+        cudaMemPool_t p = nullptr;
+        uint64_t keep = kScratchKeep;
+        if (cudaMemPoolCreate(&p, &pr) == cudaSuccess &&
+            cudaMemPoolSetAttribute(p, cudaMemPoolAttrReleaseThreshold, &keep) == cudaSuccess)
+            pools[dev] = p;
+        else
+            cudaGetLastError();  // (the default pool then)
+    }
+    return pools[dev];
+}
+}  // namespace
+
+bool scratch_alloc(void **p, size_t bytes, cudaStream_t s)
+{
+    const cudaMemPool_t pool = scratch_pool();
+    return (pool ? cudaMallocFromPoolAsync(p, bytes, pool, s) : cudaMallocAsync(p, bytes, s)) == cudaSuccess;
+}
+
+void scratch_free(void *p, cudaStream_t s) { cudaFreeAsync(p, s); }
+
+// ----------------------------------------------------------------------------
+// results and error flags of a synchronous call
+// ----------------------------------------------------------------------------
+namespace {
+struct CallResult {
+    double value;
+    unsigned flag[kErrorFlags];
+};
+struct FlagPtrs {
+    unsigned *p[kErrorFlags];
+};
+
+__global__ void k_collect(const double *value, FlagPtrs f, CallResult *out)
+{
+    if (threadIdx.x == 0 && value) out->value = *value;
+    if (threadIdx.x < kErrorFlags) out->flag[threadIdx.x] = *f.p[threadIdx.x];
+}
+
+hq_status flag_ptrs(FlagPtrs &f)
+{
+    static std::mutex mu;
+    static FlagPtrs known[64];
+    static bool have[64] = {false};
+    int dev = 0;
+    hq_status st = cuda_status("cudaGetDevice", cudaGetDevice(&dev));
+    if (st != HQ_OK) return st;
+    if (dev < 0 || dev >= 64) return HQ_ERR_ARG;
+    std::lock_guard<std::mutex> lk(mu);
+    if (!have[dev]) {
+        cudaError_t (*const get[kErrorFlags])(void **) = {pass_error_flag, batch_error_flag, expect_error_flag,
+                                                          tcz_error_flag, tc_error_flag};
+        for (int i = 0; i < kErrorFlags; ++i) {
+            void *p = nullptr;
+            if ((st = cuda_status("error flag address", get[i](&p))) != HQ_OK) return st;
+            known[dev].p[i] = static_cast<unsigned *>(p);
+        }
+        have[dev] = true;
+    }
+    f = known[dev];
+    return HQ_OK;
+}
+
+// pinned, one per host thread and device (like the staging ring); NULL on failure
+CallResult *call_result()
+{
+    static thread_local CallResult *r[64] = {nullptr};
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return nullptr;
+    if (!r[dev] && cudaHostAlloc((void **)&r[dev], sizeof(CallResult), cudaHostAllocDefault) != cudaSuccess) {
+        cudaGetLastError();
+        r[dev] = nullptr;
+    }
+    return r[dev];
+}
+
+hq_status clear_flags(const FlagPtrs &f, const unsigned *v)
+{
+    for (int i = 0; i < kErrorFlags; ++i)
+        if (v[i]) {
+            hq_status st = cuda_status("clear device error flag", cudaMemset(f.p[i], 0, sizeof(unsigned)));
+            if (st != HQ_OK) return st;
+        }
+    return HQ_OK;
+}
+}  // namespace
+
+hq_status collect_result(const double *dev_value, double *out, DeviceFlags *flags, cudaStream_t s)
+{
+    FlagPtrs f;
+    hq_status st = flag_ptrs(f);
+    if (st != HQ_OK) return st;
+    CallResult *const r = call_result();
+    if (!r) {  // no pinned memory: plain copies
+        double v = 0;
+        if (dev_value)
+            st = cuda_status("copy result", cudaMemcpyAsync(&v, dev_value, sizeof(v), cudaMemcpyDeviceToHost, s));
+        if (st == HQ_OK) st = cuda_status("sync", cudaStreamSynchronize(s));
+        if (st == HQ_OK && dev_value && out) *out = v;
+        return st;
+    }
+    k_collect<<<1, 32, 0, s>>>(dev_value, f, r);
+    if ((st = cuda_status("k_collect", cudaGetLastError())) != HQ_OK) return st;
+    if ((st = cuda_status("sync", cudaStreamSynchronize(s))) != HQ_OK) return st;
+    if (dev_value && out) *out = r->value;
+    if (flags) {
+        flags->read = true;
+        std::memcpy(flags->v, r->flag, sizeof(flags->v));
+    }
+    return HQ_OK;
+}
+
+hq_status device_error_status(cudaStream_t s, const DeviceFlags *flags)
+{
+    DeviceFlags own;
+    if (!flags || !flags->read) {
+        hq_status st = collect_result(nullptr, nullptr, &own, s);
+        if (st != HQ_OK) return st;
+        if (!own.read) return device_error_status_plain();
+        flags = &own;
+    }
+    bool any = false;
+    for (unsigned v : flags->v) any = any || v != 0;
+    if (!any) return HQ_OK;
+    FlagPtrs f;
+    hq_status st = flag_ptrs(f);
+    if (st == HQ_OK) st = clear_flags(f, flags->v);
+    return st == HQ_OK ? HQ_ERR_TIMEOUT : st;
+}
+
+hq_status device_error_status_plain()
+{
+    FlagPtrs f;
+    hq_status st = flag_ptrs(f);
+    if (st != HQ_OK) return st;
+    unsigned v[kErrorFlags];
+    bool any = false;
+    for (int i = 0; i < kErrorFlags; ++i) {
+        st = cuda_status("read device error flag", cudaMemcpy(&v[i], f.p[i], sizeof(v[i]), cudaMemcpyDeviceToHost));
+        if (st != HQ_OK) return st;
+        any = any || v[i] != 0;
+    }
+    if (!any) return HQ_OK;
+    st = clear_flags(f, v);
+    return st == HQ_OK ? HQ_ERR_TIMEOUT : st;
+}
+
 hq_status check_qubits(int n, int k, const int *qubits, int kmax)
 {
     if (!qubits) return HQ_ERR_NULL;
@@ -313,8 +480,9 @@ hq_status hq_simulate(void *state, int n, hq_dtype dt, const char *tokens, const
         if (!gates[g].matrix) return HQ_ERR_NULL;
     }
     const cudaStream_t s = (cudaStream_t)stream;
+    DeviceFlags flags;
     if (engine == HQ_ENGINE_TC_F16 || engine == HQ_ENGINE_TC_BF16) {
-        st = launch_tc_simulate(state, n, tokens, gates, G, tc_min_k, engine == HQ_ENGINE_TC_BF16, norm2_host, s);
+        st = launch_tc_simulate(state, n, tokens, gates, G, tc_min_k, engine == HQ_ENGINE_TC_BF16, norm2_host, s, &flags);
     } else {
         if ((st = launch_init(state, n, dt, tokens, 1, s)) != HQ_OK) return st;
         if ((st = hq_apply_blocks(state, n, dt, gates, G, cfg, stream)) != HQ_OK) return st;
@@ -322,11 +490,11 @@ hq_status hq_simulate(void *state, int n, hq_dtype dt, const char *tokens, const
             hq_pauli_term id;
             std::memset(&id, 0, sizeof(id));
             id.coeff = 1.0;
-            st = launch_expectation(state, n, dt, &id, 1, norm2_host, s);
+            st = launch_expectation(state, n, dt, &id, 1, norm2_host, s, &flags);
         }
     }
     if (st != HQ_OK || !norm2_host) return st;
-    return device_error_status();
+    return device_error_status(s, &flags);
 }
 
 hq_status hq_reduced_density_matrix(const void *state, int n, hq_dtype dt, const int *qubits, int k,
@@ -421,8 +589,9 @@ hq_status hq_expectation(const void *state, int n, hq_dtype dt, const hq_pauli_t
     if (st != HQ_OK) return st;
     if (!out_host) return HQ_ERR_NULL;
     if ((st = check_terms(n, terms, T)) != HQ_OK) return st;
-    if ((st = launch_expectation(state, n, dt, terms, T, out_host, (cudaStream_t)stream)) != HQ_OK) return st;
-    return device_error_status();
+    DeviceFlags flags;
+    if ((st = launch_expectation(state, n, dt, terms, T, out_host, (cudaStream_t)stream, &flags)) != HQ_OK) return st;
+    return device_error_status((cudaStream_t)stream, &flags);
 }
 
 hq_status hq_expectation_static(const void *state, int n, hq_dtype dt, const hq_pauli_term *terms, int T,
@@ -433,7 +602,7 @@ hq_status hq_expectation_static(const void *state, int n, hq_dtype dt, const hq_
     if (!out_host) return HQ_ERR_NULL;
     if ((st = check_terms(n, terms, T)) != HQ_OK) return st;
     if ((st = launch_expectation_static(state, n, dt, terms, T, out_host, (cudaStream_t)stream)) != HQ_OK) return st;
-    return device_error_status();
+    return device_error_status_plain();
 }
 
 }  // extern "C"

@@ -77,7 +77,7 @@ static hq_status run_dm_expectation(const void *rho, int n, const hq_pauli_term 
                               ((int64_t(1) << n) + kDmThreads - 1) / kDmThreads);
     const int nparts = grid * nchunks;
     double *scratch = nullptr;
-    if (injected_alloc_failure() || cudaMallocAsync((void **)&scratch, sizeof(double) * (size_t(nparts) + 1), s) != cudaSuccess)
+    if (injected_alloc_failure() || !scratch_alloc((void **)&scratch, sizeof(double) * (size_t(nparts) + 1), s))
         return HQ_ERR_ALLOC;
     hq_status st = HQ_OK;
     for (int c = 0; c < nchunks && st == HQ_OK; ++c) {
@@ -104,13 +104,8 @@ static hq_status run_dm_expectation(const void *rho, int n, const hq_pauli_term 
         k_dm_final<<<1, kDmThreads, 0, s>>>(scratch, nparts, scratch + nparts);
         st = cuda_status("k_dm_final", cudaGetLastError());
     }
-    double out = 0;
-    if (st == HQ_OK)
-        st = cuda_status("copy result", cudaMemcpyAsync(&out, scratch + nparts, sizeof(double),
-                                                        cudaMemcpyDeviceToHost, s));
-    cudaFreeAsync(scratch, s);
-    if (st == HQ_OK) st = cuda_status("sync", cudaStreamSynchronize(s));
-    if (st == HQ_OK) *out_host = out;
+    if (st == HQ_OK) st = collect_result(scratch + nparts, out_host, nullptr, s);
+    scratch_free(scratch, s);
     return st;
 }
 

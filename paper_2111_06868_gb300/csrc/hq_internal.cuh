@@ -33,6 +33,12 @@ hq_status upload_async(void *dst, const void *src, size_t bytes, cudaStream_t s)
 // event dst_ready (recorded on s once dst is allocated; NULL: no wait), with
 // s made to wait for it: it does not queue behind the kernels already on s.
 hq_status upload_side(void *dst, const void *src, size_t bytes, cudaStream_t s, cudaEvent_t dst_ready);
+// Device scratch of a call: stream-ordered, from a pool that the library owns per
+// device (up to 16 MB stay mapped between calls: the default pool gives
+// everything back at each synchronisation, and mapping it again took 0.2 ms of a
+// call).  False when the memory cannot be had.
+bool scratch_alloc(void **p, size_t bytes, cudaStream_t s);
+void scratch_free(void *p, cudaStream_t s);
 // A per-thread, per-device event for one call's orderings (NULL on failure).
 cudaEvent_t call_event();
 // resident CTAs per SM of `fn` (sets the dynamic shared-memory attribute when
@@ -257,9 +263,33 @@ hq_status launch_rdm(const void *state, int n, hq_dtype dt, const int *qubits, i
 hq_status run_trajectory(void *state, int n, hq_dtype dt, const hq_noisy_op *ops, int nops, const double *u,
                          int *chosen, const hq_config *cfg, cudaStream_t s);
 
+// The device error flags (a bounded wait ran out) as one read found them.
+constexpr int kErrorFlags = 5;
+struct DeviceFlags {
+    bool read = false;
+    unsigned v[kErrorFlags] = {0, 0, 0, 0, 0};
+};
+// Synchronises s: the double at dev_value (NULL: none) into *out and the error
+// flags into *flags (NULL: not wanted), by one kernel that writes pinned host
+// memory -- one launch and one wait instead of a copy for the value and one for each flag.
+hq_status collect_result(const double *dev_value, double *out, DeviceFlags *flags, cudaStream_t s);
+// HQ_ERR_TIMEOUT (and clears the flags) if a bounded device-side wait ran out
+// since the last call: by what `flags` holds when it was read, else by reading
+// the flags after the work on s; synchronous.
+hq_status device_error_status(cudaStream_t s, const DeviceFlags *flags = nullptr);
+// the same by plain copies, for callers that must not allocate (pinned memory included)
+hq_status device_error_status_plain();
+// device addresses of the flags
+cudaError_t tc_error_flag(void **p);
+cudaError_t pass_error_flag(void **p);
+cudaError_t batch_error_flag(void **p);
+cudaError_t expect_error_flag(void **p);
+cudaError_t tcz_error_flag(void **p);
+
 // expectation (k_reduce.cu)
+// (flags: also the device error flags, where the sum needed a kernel)
 hq_status launch_expectation(const void *state, int n, hq_dtype dt, const hq_pauli_term *terms, int T,
-                             double *out_host, cudaStream_t s);
+                             double *out_host, cudaStream_t s, DeviceFlags *flags = nullptr);
 
 // tensor-core block engine (k_tc.cu); complex64 only, k in {5, 6}
 hq_status launch_tc_block(void *state, int n, int k, const int *qubits, const double *matrix, int64_t nstates,
@@ -268,9 +298,6 @@ hq_status launch_tc_block(void *state, int n, int k, const int *qubits, const do
 hq_status launch_expectation_static(const void *state, int n, hq_dtype dt, const hq_pauli_term *terms, int T,
                                     double *out_host, cudaStream_t s);
 
-// HQ_ERR_TIMEOUT (and clears the flag) if a bounded device-side wait ran out
-// since the last call; synchronous.
-hq_status device_error_status();
 // Tensor-core engine over a list of gates: every gate with tc_min_k <= k
 // (k >= 4, not diagonal) runs on k_tc, the others through launch_gate; all
 // split matrices are prepared on the host and copied in one transfer.
@@ -280,7 +307,7 @@ hq_status launch_tc_blocks(void *state, int n, const hq_gate *gates, int G, int 
 // is set, the FP64 squared norm of the result (synchronous then): the first
 // and last blocks fold the initialisation and the norm in when they run on k_tc.
 hq_status launch_tc_simulate(void *state, int n, const char *tokens, const hq_gate *gates, int G, int tc_min_k,
-                             int split_bf16, double *norm2_host, cudaStream_t s);
+                             int split_bf16, double *norm2_host, cudaStream_t s, DeviceFlags *flags);
 
 // Tile passes (k_pass.cu).  One pass holds a 13-bit tile that contains the 7
 // lowest physical bits, applies up to two fused blocks to it and permutes its
@@ -293,20 +320,11 @@ struct PassPlanEntry {
 };
 void plan_passes(int n, const hq_gate *gates, int G, int max_blocks, std::vector<PassPlanEntry> &plan);
 hq_status launch_tc_passes(void *state, int n, const hq_gate *gates, int G, int max_blocks, cudaStream_t s);
-hq_status pass_error_status();
-// HQ_ERR_TIMEOUT (and the flag cleared) if a batch run's scheduler gave up
-// (k_batch.cu); device_error_status() checks it too.
-hq_status batch_error_status();
-// HQ_ERR_TIMEOUT (and the flag cleared) if a staged expectation pass gave up
-// a bounded wait (k_expect_reg.cu); device_error_status() checks it too.
-hq_status expect_error_status();
 // complex128 blocks of k = 3, 4 on the tensor cores (k_tcz.cu): dense blocks
-// on n >= 11 qubits; 3-qubit blocks run widened to 4.  The error status as
-// above for its bounded waits.
+// on n >= 11 qubits; 3-qubit blocks run widened to 4.
 bool tcz_eligible(int n, int k, const double *mat);
 hq_status launch_tcz_block(void *state, int n, int k, const int *qubits, const double *mat, int64_t nstates,
                            cudaStream_t s);
-hq_status tcz_error_status();
 
 // validation helpers (hq_api.cu)
 hq_status check_qubits(int n, int k, const int *qubits, int kmax);

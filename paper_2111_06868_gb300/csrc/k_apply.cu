@@ -951,11 +951,11 @@ static hq_status run_block(void *state, int n, const int *qubits, const double *
         hm[i].y = R(mat[2 * i + 1]);
     }
     T2 *dm = nullptr;
-    if (injected_alloc_failure() || cudaMallocAsync((void **)&dm, sizeof(T2) * D * D, s) != cudaSuccess)
+    if (injected_alloc_failure() || !scratch_alloc((void **)&dm, sizeof(T2) * D * D, s))
         return HQ_ERR_ALLOC;
     hq_status st = upload_async(dm, hm.data(), sizeof(T2) * D * D, s);
     if (st != HQ_OK) {
-        cudaFreeAsync(dm, s);
+        scratch_free(dm, s);
         return st;
     }
     const size_t smem = sizeof(T2) * (size_t(D * D) + (size_t(1) << g.L));
@@ -963,7 +963,7 @@ static hq_status run_block(void *state, int n, const int *qubits, const double *
     const int grid = grid_for(fn, kThreads, smem, g.total_tiles);
     k_block<R, K><<<grid, kThreads, smem, s>>>(g, dm, (T2 *)state);
     st = cuda_status("k_block", cudaGetLastError());
-    cudaFreeAsync(dm, s);
+    scratch_free(dm, s);
     return st;
 }
 

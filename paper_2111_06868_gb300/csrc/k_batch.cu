@@ -342,19 +342,7 @@ __global__ void __launch_bounds__(kBThreads) k_batch(const BatchParams p)
     }
 }
 
-hq_status batch_error_status()
-{
-    unsigned int v = 0;
-    cudaError_t e = cudaMemcpyFromSymbol(&v, g_batch_error, sizeof(v));
-    if (e != cudaSuccess) return cuda_status("read batch error flag", e);
-    if (v) {
-        const unsigned int zero = 0;
-        e = cudaMemcpyToSymbol(g_batch_error, &zero, sizeof(zero));
-        if (e != cudaSuccess) return cuda_status("clear batch error flag", e);
-        return HQ_ERR_TIMEOUT;
-    }
-    return HQ_OK;
-}
+cudaError_t batch_error_flag(void **p) { return cudaGetSymbolAddress(p, g_batch_error); }
 
 static size_t align_up256(size_t v) { return (v + 255) & ~size_t(255); }
 
@@ -659,7 +647,7 @@ extern "C" hq_status hq_batch_latencies(hq_batch *b, void *stream, float *latenc
                             cudaMemcpyDeviceToHost, s));
     HQ_CUDA(cudaMemcpyAsync(&t0, b->ws + b->off_t0, sizeof(t0), cudaMemcpyDeviceToHost, s));
     HQ_CUDA(cudaStreamSynchronize(s));
-    hq_status st = device_error_status();
+    hq_status st = device_error_status(s);
     if (st != HQ_OK) return st;
     unsigned long long mx = t0;
     for (int c = 0; c < b->C; ++c) {

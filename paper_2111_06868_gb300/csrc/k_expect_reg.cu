@@ -362,19 +362,7 @@ bool plan_expect_reg(int n, int H, const int *high_bits, const std::vector<EvInR
     return true;
 }
 
-hq_status expect_error_status()
-{
-    unsigned int v = 0;
-    cudaError_t e = cudaMemcpyFromSymbol(&v, g_expect_error, sizeof(v));
-    if (e != cudaSuccess) return cuda_status("read expectation error flag", e);
-    if (v) {
-        const unsigned int zero = 0;
-        e = cudaMemcpyToSymbol(g_expect_error, &zero, sizeof(zero));
-        if (e != cudaSuccess) return cuda_status("clear expectation error flag", e);
-        return HQ_ERR_TIMEOUT;
-    }
-    return HQ_OK;
-}
+cudaError_t expect_error_flag(void **p) { return cudaGetSymbolAddress(p, g_expect_error); }
 
 hq_status launch_expect_reg(const void *state, hq_dtype dt, const ErParams &p, int grid, double *partials,
                             cudaStream_t s)

@@ -160,7 +160,7 @@ static hq_status run_rdm(const void *state, int n, const int *qubits, double *ou
     const int width = 2 * NE;
     double *scratch = nullptr;
     if (injected_alloc_failure() ||
-        cudaMallocAsync((void **)&scratch, sizeof(double) * (size_t(grid) + 1) * width, s) != cudaSuccess)
+        !scratch_alloc((void **)&scratch, sizeof(double) * (size_t(grid) + 1) * width, s))
         return HQ_ERR_ALLOC;
     hq_status rc = rdm_partials<R, K>(state, n, qubits, scratch, s);
     double *out_dev = scratch + size_t(grid) * width;
@@ -172,7 +172,7 @@ static hq_status run_rdm(const void *state, int n, const int *qubits, double *ou
     if (rc == HQ_OK)
         rc = cuda_status("copy result",
                          cudaMemcpyAsync(tri.data(), out_dev, sizeof(double) * width, cudaMemcpyDeviceToHost, s));
-    cudaFreeAsync(scratch, s);
+    scratch_free(scratch, s);
     if (rc == HQ_OK) rc = cuda_status("sync", cudaStreamSynchronize(s));
     if (rc != HQ_OK) return rc;
     int e = 0;
@@ -1082,12 +1082,12 @@ hq_status run_trajectory(void *state, int n, hq_dtype dt, const hq_noisy_op *ops
     const size_t bytes = nd * sizeof(double) + sizeof(int) * (dev.size() + 1);
     char *ws = nullptr;
     if (!dev.empty()) {
-        if (injected_alloc_failure() || cudaMallocAsync((void **)&ws, bytes, s) != cudaSuccess) return HQ_ERR_ALLOC;
+        if (injected_alloc_failure() || !scratch_alloc((void **)&ws, bytes, s)) return HQ_ERR_ALLOC;
         hq_status cs = upload_async(ws, hostbuf.data(), sizeof(double) * hostbuf.size(), s);
         if (cs == HQ_OK)
             cs = cuda_status("clear chosen", cudaMemsetAsync(ws + nd * sizeof(double), 0, sizeof(int) * (dev.size() + 1), s));
         if (cs != HQ_OK) {
-            cudaFreeAsync(ws, s);
+            scratch_free(ws, s);
             return cs;
         }
     }
@@ -1219,7 +1219,7 @@ hq_status run_trajectory(void *state, int n, hq_dtype dt, const hq_noisy_op *ops
     if (st == HQ_OK)
         st = cuda_status("copy chosen", cudaMemcpyAsync(back.data(), chosen_dev, sizeof(int) * back.size(),
                                                         cudaMemcpyDeviceToHost, s));
-    cudaFreeAsync(ws, s);
+    scratch_free(ws, s);
     if (st == HQ_OK) st = cuda_status("sync", cudaStreamSynchronize(s));
     if (st != HQ_OK) return st;
     if (back[dev.size()]) {

@@ -866,7 +866,7 @@ hq_status launch_tc_passes(void *state, int n, const hq_gate *gates, int G, int 
     }
     uint4 *dmat = nullptr;
     const size_t bytes = hb.size() * sizeof(uint16_t);
-    if (injected_alloc_failure() || cudaMallocAsync((void **)&dmat, bytes, s) != cudaSuccess) return HQ_ERR_ALLOC;
+    if (injected_alloc_failure() || !scratch_alloc((void **)&dmat, bytes, s)) return HQ_ERR_ALLOC;
     hq_status st = upload_async(dmat, hb.data(), bytes, s);
     bi = 0;
     for (size_t pi = 0; pi < plan.size() && st == HQ_OK; ++pi) {
@@ -890,21 +890,10 @@ hq_status launch_tc_passes(void *state, int n, const hq_gate *gates, int G, int 
         }
         bi += size_t(pl.nb);
     }
-    cudaFreeAsync(dmat, s);
+    scratch_free(dmat, s);
     return st;
 }
 
-hq_status pass_error_status()
-{
-    unsigned int v = 0;
-    cudaError_t e = cudaMemcpyFromSymbol(&v, g_pass_error, sizeof(v));
-    if (e != cudaSuccess) return cuda_status("read pass error flag", e);
-    if (v) {
-        const unsigned int zero = 0;
-        cudaMemcpyToSymbol(g_pass_error, &zero, sizeof(zero));
-        return HQ_ERR_TIMEOUT;
-    }
-    return HQ_OK;
-}
+cudaError_t pass_error_flag(void **p) { return cudaGetSymbolAddress(p, g_pass_error); }
 
 }  // namespace hq

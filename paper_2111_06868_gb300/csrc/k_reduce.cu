@@ -653,7 +653,7 @@ static hq_status launch_tiled(const void *state, int n, hq_dtype dt, const std::
 }
 
 hq_status launch_expectation(const void *state, int n, hq_dtype dt, const hq_pauli_term *terms, int T,
-                             double *out_host, cudaStream_t s)
+                             double *out_host, cudaStream_t s, DeviceFlags *flags)
 {
     // several X-mask groups: one read of the state per tile pass instead of one per group
     if (n >= 13 && T > 0) {
@@ -671,15 +671,11 @@ hq_status launch_expectation(const void *state, int n, hq_dtype dt, const hq_pau
             const int grid = 3 * sm_count();
             double *scratch = nullptr;
             const size_t nd = 1 + passes.size() * size_t(grid);
-            if (injected_alloc_failure() || cudaMallocAsync((void **)&scratch, sizeof(double) * nd, s) != cudaSuccess)
+            if (injected_alloc_failure() || !scratch_alloc((void **)&scratch, sizeof(double) * nd, s))
                 return HQ_ERR_ALLOC;
             st = launch_tiled(state, n, dt, passes, grid, scratch, s);
-            double result = 0;
-            if (st == HQ_OK)
-                st = cuda_status("copy result", cudaMemcpyAsync(&result, scratch, sizeof(double), cudaMemcpyDeviceToHost, s));
-            cudaFreeAsync(scratch, s);
-            if (st == HQ_OK) st = cuda_status("sync", cudaStreamSynchronize(s));
-            if (st == HQ_OK) *out_host = result;
+            if (st == HQ_OK) st = collect_result(scratch, out_host, flags, s);
+            scratch_free(scratch, s);
             return st;
         }
     }
@@ -705,7 +701,7 @@ hq_status launch_expectation(const void *state, int n, hq_dtype dt, const hq_pau
     }
     const size_t npart = size_t(groups.size()) * gx;
     double *scratch = nullptr;
-    if (injected_alloc_failure() || cudaMallocAsync((void **)&scratch, sizeof(double) * (npart + 1), s) != cudaSuccess)
+    if (injected_alloc_failure() || !scratch_alloc((void **)&scratch, sizeof(double) * (npart + 1), s))
         return HQ_ERR_ALLOC;
     hq_status rc = HQ_OK;
     for (auto &ch : chunks) {
@@ -734,12 +730,8 @@ hq_status launch_expectation(const void *state, int n, hq_dtype dt, const hq_pau
         k_expect_final<<<1, kRedThreads, 0, s>>>(scratch, int(groups.size()), gx, scratch + npart);
         rc = cuda_status("k_expect_final", cudaGetLastError());
     }
-    double result = 0;
-    if (rc == HQ_OK) rc = cuda_status("copy result", cudaMemcpyAsync(&result, scratch + npart, sizeof(double),
-                                                                       cudaMemcpyDeviceToHost, s));
-    cudaFreeAsync(scratch, s);
-    if (rc == HQ_OK) rc = cuda_status("sync", cudaStreamSynchronize(s));
-    if (rc == HQ_OK) *out_host = result;
+    if (rc == HQ_OK) rc = collect_result(scratch + npart, out_host, flags, s);
+    scratch_free(scratch, s);
     return rc;
 }
 

@@ -865,7 +865,7 @@ static hq_status launch_tc_list(void *state, int n, const hq_gate *gates, int G,
     const size_t norm_off = bytes, norm_slots = size_t(sm_count()) * 4 * 8;
     if (norm) bytes += norm_slots * sizeof(double);
     char *dmat = nullptr;
-    if (bytes && (injected_alloc_failure() || cudaMallocAsync((void **)&dmat, bytes, s) != cudaSuccess))
+    if (bytes && (injected_alloc_failure() || !scratch_alloc((void **)&dmat, bytes, s)))
         return HQ_ERR_ALLOC;
     hq_status st = HQ_OK;
     double *norm_part = norm ? reinterpret_cast<double *>(dmat + norm_off) : nullptr;
@@ -927,7 +927,7 @@ static hq_status launch_tc_list(void *state, int n, const hq_gate *gates, int G,
         st = cuda_status("read norm partials", cudaMemcpyAsync(ex->norm_slots->data(), norm_part,
                                                                norm_slots * sizeof(double), cudaMemcpyDeviceToHost, s));
     }
-    if (dmat) cudaFreeAsync(dmat, s);
+    if (dmat) scratch_free(dmat, s);
     return st;
 }
 
@@ -941,7 +941,7 @@ static hq_status launch_tc_list(void *state, int n, const hq_gate *gates, int G,
 // Otherwise the initialisation kernel and the streaming norm run as separate
 // passes.
 hq_status launch_tc_simulate(void *state, int n, const char *tokens, const hq_gate *gates, int G, int tc_min_k,
-                             int split_bf16, double *norm2_host, cudaStream_t s)
+                             int split_bf16, double *norm2_host, cudaStream_t s, DeviceFlags *flags)
 {
     TcListExtras ex;
     int m = 0;
@@ -972,9 +972,9 @@ hq_status launch_tc_simulate(void *state, int n, const char *tokens, const hq_ga
         hq_pauli_term id;
         std::memset(&id, 0, sizeof(id));
         id.coeff = 1.0;
-        return launch_expectation(state, n, HQ_C64, &id, 1, norm2_host, s);
+        return launch_expectation(state, n, HQ_C64, &id, 1, norm2_host, s, flags);
     }
-    if ((st = cuda_status("simulate sync", cudaStreamSynchronize(s))) != HQ_OK) return st;
+    if ((st = collect_result(nullptr, nullptr, flags, s)) != HQ_OK) return st;
     double sum = 0.0;
     for (double v : slots) sum += v;
     *norm2_host = sum;
@@ -998,25 +998,6 @@ hq_status launch_tc_blocks(void *state, int n, const hq_gate *gates, int G, int 
     return launch_tc_list(state, n, gates, G, tc_min_k, split_bf16, 1, s);
 }
 
-hq_status device_error_status()
-{
-    const hq_status ps = pass_error_status();
-    if (ps != HQ_OK) return ps;
-    const hq_status bs = batch_error_status();
-    if (bs != HQ_OK) return bs;
-    const hq_status es = expect_error_status();
-    if (es != HQ_OK) return es;
-    const hq_status zs = tcz_error_status();
-    if (zs != HQ_OK) return zs;
-    unsigned int v = 0;
-    cudaError_t e = cudaMemcpyFromSymbol(&v, g_device_error, sizeof(v));
-    if (e != cudaSuccess) return cuda_status("read device error flag", e);
-    if (v) {
-        const unsigned int zero = 0;
-        cudaMemcpyToSymbol(g_device_error, &zero, sizeof(zero));
-        return HQ_ERR_TIMEOUT;
-    }
-    return HQ_OK;
-}
+cudaError_t tc_error_flag(void **p) { return cudaGetSymbolAddress(p, g_device_error); }
 
 }  // namespace hq

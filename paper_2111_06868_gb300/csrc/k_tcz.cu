@@ -517,7 +517,7 @@ hq_status launch_tcz_block(void *state, int n, int k, const int *qubits, const d
     p.w24 = 1u << 24;
     const size_t bytes = bh.size() * sizeof(uint16_t);
     char *dmat = nullptr;
-    if (injected_alloc_failure() || cudaMallocAsync((void **)&dmat, bytes, s) != cudaSuccess) return HQ_ERR_ALLOC;
+    if (injected_alloc_failure() || !scratch_alloc((void **)&dmat, bytes, s)) return HQ_ERR_ALLOC;
     hq_status st = upload_async(dmat, bh.data(), bytes, s);
     if (st == HQ_OK) {
         p.bmat = reinterpret_cast<const uint4 *>(dmat);
@@ -529,21 +529,10 @@ hq_status launch_tcz_block(void *state, int n, int k, const int *qubits, const d
         k_tcz<<<grid, kZThreads, smem, s>>>(p, (double2 *)state);
         st = cuda_status("k_tcz", cudaGetLastError());
     }
-    cudaFreeAsync(dmat, s);
+    scratch_free(dmat, s);
     return st;
 }
 
-hq_status tcz_error_status()
-{
-    unsigned int v = 0;
-    cudaError_t e = cudaMemcpyFromSymbol(&v, g_tcz_error, sizeof(v));
-    if (e != cudaSuccess) return cuda_status("read k_tcz error flag", e);
-    if (v) {
-        const unsigned int zero = 0;
-        cudaMemcpyToSymbol(g_tcz_error, &zero, sizeof(zero));
-        return HQ_ERR_TIMEOUT;
-    }
-    return HQ_OK;
-}
+cudaError_t tcz_error_flag(void **p) { return cudaGetSymbolAddress(p, g_tcz_error); }
 
 }  // namespace hq
