@@ -189,3 +189,25 @@ def test_adjoint_argument_errors(hq):
     small = torch.empty(64, dtype=torch.uint8, device="cuda")
     with pytest.raises(hq.HQError, match="CAPACITY"):
         hq.hq_adjoint_grad(circ, H, th, dtype="complex128", workspace=small)
+
+
+@pytest.mark.parametrize("batch", [1, 3, 4, 5, 8, 9, 17])
+@pytest.mark.parametrize("dt", ["complex64", "complex128"])
+def test_hamiltonians_with_shared_masks_over_batches(hq, dt, batch):
+    """lambda = H phi is formed for several parameter sets at once, terms with one
+    X mask together: sums with repeated masks, Y factors (imaginary weights),
+    the identity, batches that leave a remainder."""
+    n = 7
+    circ = C.ansatz(n, 2)
+    H = [(0.7, ()), (1.0, ((0, "Z"), (3, "Z"))), (-0.4, ((2, "Z"),)), (0.5, ((1, "X"),)), (0.3, ((1, "Y"),)),
+         (-0.8, ((1, "X"), (4, "Z"))), (0.6, ((1, "Y"), (5, "Z"), (6, "Z"))), (0.2, ((0, "Y"), (2, "Y"))),
+         (0.9, ((0, "X"), (2, "X"))), (-0.1, ((0, "Y"), (2, "X"))), (0.25, ((6, "X"),)), (0.15, ((0, "Z"),))]
+    th = C.ansatz_params(circ.n_params, batch, 11)
+    e, g = hq.hq_adjoint_grad(circ, H, th, dtype=dt)
+    scale = sum(abs(c) for c, _ in H)
+    for b in range(batch):
+        we, wg = oracle.adjoint_grad(circ, H, th[b])
+        # complex64: ~60 gates, each rounding the state by a few 2^-24
+        tol = (1e-10 if dt == "complex128" else 2e-5) * scale
+        assert abs(e[b] - we) <= tol
+        assert np.abs(g[b] - wg).max() <= tol
