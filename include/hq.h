@@ -436,10 +436,12 @@ hq_status hq_apply_gate(void *state, int n, hq_dtype dt, const int *qubits, int 
  * see hq_plan_passes.  It moves qubits between bit positions while it runs and
  * restores the caller's order before it returns (stream order).
  * HQ_ENGINE_AUTO and HQ_ENGINE_CUDA_CORE apply runs of one- and two-qubit and
- * diagonal gates many at a time, each tile of the state read and written once
- * per pass (gates with disjoint qubits may swap); a product with an exactly
- * zero real or imaginary part of a matrix entry is left out there, so an
- * infinity or NaN among the amplitudes spreads only through nonzero parts.
+ * diagonal gates (complex64: of up to 4 qubits) many at a time, each tile of the
+ * state read and written once per pass (gates with disjoint qubits may swap; on
+ * large complex64 states a pass's gates are multiplied, in double, into blocks of 3 or
+ * 4 qubits first); a product with an exactly zero real or imaginary part of a
+ * matrix entry may be left out there, so an infinity or NaN among the amplitudes
+ * may spread only through nonzero parts.
  * Errors: as hq_apply_gate, plus HQ_ERR_ARG (G < 0 or unknown engine).
  * On HQ_ERR_ALLOC the state is left as follows: the tensor-core engines and
  * HQ_ENGINE_TC_PASS take their one scratch buffer before enqueueing any

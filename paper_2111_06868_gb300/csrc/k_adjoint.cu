@@ -130,11 +130,11 @@ struct HamTerm {
     double wr, wi;   // coeff * (-i)^#Y
     float wrf, wif;  // the same in FP32 (complex64 states: no FP64 conversion per amplitude)
     int last;        // the last of its run of terms with one X mask
-    int imag;        // (last term of a run) a weight of the run has an imaginary part
+    int imag;        // the weight has an imaginary part
 };
 constexpr int kMaxHamTerms = 128;
 struct HamParams {
-    int T, n, batch;  // terms sorted by X mask
+    int T, n, batch;
     HamTerm t[kMaxHamTerms];
 };
 
@@ -146,12 +146,14 @@ __device__ __forceinline__ double flip(double w, int odd)
 }
 
 // lambda_b = H phi_b and partial <phi_b|lambda_b>; grid (x, ceil(batch / BC)).
-// A run of terms with one X mask needs one amplitude per state, times the sum of
-// the terms' signed weights; that sum depends on the index x only, so a thread
-// forms it once for BC parameter sets (integer sign flips; complex128: FP64
-// additions cost 64 cycles of an SM quarter each).  With a load, a popcount and
-// a complex multiply-add per term and state, n = 20: batch 64 complex64 4.43
-// ms, batch 16 complex128 7.12 ms, against 1 GB / 0.5 GB of traffic.
+// Consecutive terms with one X mask (a run) read one amplitude per state, and a
+// term's sign depends on the index x only: a thread forms it once (integer sign
+// flips) for BC parameter sets.  complex64: one multiply-add per term, in the
+// caller's order (FP32 sums keep their rounding).  complex128: terms sorted by X
+// mask, the weights of a run summed first (an FP64 instruction costs 64 cycles
+// of an SM quarter; weights once per BC sets instead of products per set).
+// With a load, a popcount and a complex multiply-add per term and state, n = 20, 39 terms: batch 64 complex64 4.43
+// ms, batch 16 complex128 7.12 ms, against 1 GB / 0.5 GB of traffic; this: HAM64 and 2.68 ms.
 template <typename R, int BC>
 __global__ void __launch_bounds__(kAdjThreads) k_ham(const __grid_constant__ HamParams p,
                                                      const typename C2<R>::type *__restrict__ phi,
@@ -173,33 +175,54 @@ __global__ void __launch_bounds__(kAdjThreads) k_ham(const __grid_constant__ Ham
         for (int b = 0; b < BC; ++b) out[b].x = out[b].y = 0;
         for (int t = 0; t < p.T;) {
             const T2 *const from = sp + (x ^ int64_t(p.t[t].xm));
-            T2 w;
-            w.x = w.y = 0;
-            bool last = false, imag = false;
-            while (!last) {
-                const HamTerm &h = p.t[t++];
-                const int odd = __popcll(uint64_t(x) & h.zm) & 1;
-                if constexpr (sizeof(R) == 4) {
-                    w.x += flip(h.wrf, odd);
-                    w.y += flip(h.wif, odd);
-                } else {
-                    w.x += flip(h.wr, odd);
-                    if (h.wi != 0.0) w.y += flip(h.wi, odd);
-                }
-                last = h.last != 0;
-                imag = h.imag != 0;
-            }
-            if (imag) {
+            bool last = false;
+            if constexpr (sizeof(R) == 4) {
+                T2 a[BC];
 #pragma unroll
                 for (int b = 0; b < BC; ++b)
-                    if (b < nb) cmac(out[b], w, from[b * dim]);
+                    if (b < nb) a[b] = from[b * dim];
+                while (!last) {
+                    const HamTerm &h = p.t[t++];
+                    const int odd = __popcll(uint64_t(x) & h.zm) & 1;
+                    T2 w;
+                    w.x = flip(h.wrf, odd);
+                    w.y = flip(h.wif, odd);
+                    if (h.wif == 0.f) {
+#pragma unroll
+                        for (int b = 0; b < BC; ++b)
+                            if (b < nb) {
+                                out[b].x = fmaf(w.x, a[b].x, out[b].x);
+                                out[b].y = fmaf(w.x, a[b].y, out[b].y);
+                            }
+                    } else {
+#pragma unroll
+                        for (int b = 0; b < BC; ++b)
+                            if (b < nb) cmac(out[b], w, a[b]);
+                    }
+                    last = h.last != 0;
+                }
             } else {
+                T2 w;
+                w.x = w.y = 0;
+                bool imag = false;
+                while (!last) {
+                    const HamTerm &h = p.t[t++];
+                    const int odd = __popcll(uint64_t(x) & h.zm) & 1;
+                    w.x += flip(h.wr, odd);
+                    if (h.imag) w.y += flip(h.wi, odd);
+                    imag = imag || h.imag != 0;
+                    last = h.last != 0;
+                }
 #pragma unroll
                 for (int b = 0; b < BC; ++b)
                     if (b < nb) {
                         const T2 a = from[b * dim];
-                        out[b].x = fma(w.x, a.x, out[b].x);
-                        out[b].y = fma(w.x, a.y, out[b].y);
+                        if (imag) {
+                            cmac(out[b], w, a);
+                        } else {
+                            out[b].x = fma(w.x, a.x, out[b].x);
+                            out[b].y = fma(w.x, a.y, out[b].y);
+                        }
                     }
             }
         }
@@ -411,21 +434,26 @@ extern "C" hq_status hq_adjoint_grad(int n, hq_dtype dt, const hq_op *ops, int G
     void *lam = static_cast<char *>(phi) + state_bytes;
     double *epart = part + size_t(G) * batch * nbx;
     {
-        std::stable_sort(hp.t, hp.t + T, [](const HamTerm &a, const HamTerm &b) { return a.xm < b.xm; });
-        bool imag = false;
+        if (dt == HQ_C128)
+            std::stable_sort(hp.t, hp.t + T, [](const HamTerm &a, const HamTerm &b) { return a.xm < b.xm; });
         for (int t = 0; t < T; ++t) {
-            imag = imag || hp.t[t].wi != 0.0;
             hp.t[t].last = t + 1 == T || hp.t[t + 1].xm != hp.t[t].xm;
-            hp.t[t].imag = imag;
-            if (hp.t[t].last) imag = false;
+            hp.t[t].imag = hp.t[t].wi != 0.0;
         }
         hp.batch = batch;
+        // several sets per thread only where that still leaves a CTA for every SM
         const int bc = dt == HQ_C64 ? kHamBatch64 : kHamBatch128;
-        dim3 grid(nbx, (batch + bc - 1) / bc);
-        if (dt == HQ_C64)
-            k_ham<float, kHamBatch64><<<grid, kAdjThreads, 0, s>>>(hp, (const float2 *)phi, (float2 *)lam, epart);
-        else
-            k_ham<double, kHamBatch128><<<grid, kAdjThreads, 0, s>>>(hp, (const double2 *)phi, (double2 *)lam, epart);
+        const bool several = int64_t(nbx) * ((batch + bc - 1) / bc) >= sm_count();
+        const dim3 grid(nbx, several ? (batch + bc - 1) / bc : batch);
+        if (dt == HQ_C64) {
+            const float2 *const in = (const float2 *)phi;
+            if (several) k_ham<float, kHamBatch64><<<grid, kAdjThreads, 0, s>>>(hp, in, (float2 *)lam, epart);
+            else k_ham<float, 1><<<grid, kAdjThreads, 0, s>>>(hp, in, (float2 *)lam, epart);
+        } else {
+            const double2 *const in = (const double2 *)phi;
+            if (several) k_ham<double, kHamBatch128><<<grid, kAdjThreads, 0, s>>>(hp, in, (double2 *)lam, epart);
+            else k_ham<double, 1><<<grid, kAdjThreads, 0, s>>>(hp, in, (double2 *)lam, epart);
+        }
         HQ_CUDA(cudaGetLastError());
     }
 

@@ -28,7 +28,9 @@
 // moves that a packed FMA's crosswise operand needs and shared-memory addresses; DRAM 16 %), complex128 the FP64 pipe.
 // Tried and slower, n=28 circuit (785 gates): 8 amplitudes per thread 123 ms, scalar FMAs 120 ms, packed real and
 // scalar imaginary products 94 ms, 512 threads at 64 registers 102 ms, two CTAs per SM 95 ms, against 87 ms.
-// Per-gate circuits, against one launch per gate: n=28 complex64 depth 20 fSim 528 -> 87 ms (26 passes), n=20
+// From 23 qubits on (and for 3- and 4-qubit gates) a complex64 pass may instead fuse its gates into dense blocks
+// (k_block_pass.cu); the kind that does more work per time is chosen pass by pass.
+// Per-gate circuits, against one launch per gate: n=28 complex64 depth 20 fSim 528 -> 87 ms (55 in blocks), n=20
 // depth 16 CZ 1.53 -> 0.25 ms of device time, n=12 complex128 depth 10 1.06 -> 0.24 ms.
 #include <algorithm>
 #include <cmath>
@@ -36,6 +38,7 @@
 #include <new>
 #include <vector>
 
+#include "hq_block_pass.cuh"
 #include "hq_cp_async.cuh"
 #include "hq_internal.cuh"
 
@@ -58,7 +61,8 @@ enum OpKind : uint8_t {
     OP_U2 = 1,    // dense 4 x 4 on the register position pair var
     OP_D2 = 2,    // a phase for each value of the pair var
     OP_PH = 3,    // a phase where all controls are 1 (var: controls among the register positions)
-    OP_DG = 4     // a diagonal gate of k qubits by its table
+    OP_DG = 4,    // a diagonal gate of k qubits by its table
+    OP_BLK = 5    // a 3- or 4-qubit gate that only a pass of dense blocks takes (k_block_pass.cu)
 };
 
 // zero parts of a 2 x 2 matrix (sqrt(Y), H, RY: real; sqrt(X), RX: real diagonal, imaginary off it; sqrt(W): real
@@ -512,6 +516,8 @@ __global__ void __launch_bounds__(kRunThreads, 3) k_runs(const __grid_constant__
 // ----------------------------------------------------------------------------
 // planning (host)
 // ----------------------------------------------------------------------------
+constexpr uint64_t kNever = uint64_t(1) << 63;  // in Item::need: not for register runs
+
 // One gate as the planner sees it.
 struct Item {
     OpKind kind;
@@ -522,7 +528,7 @@ struct Item {
     uint8_t flags;
     bool swap;          // OP_D2: exchange the two qubits first
     uint16_t keep;      // OP_U2: bit 4 r + c set where the entry is not an exact zero
-    uint64_t all, need;
+    uint64_t all, need; // flat bits; those that a register run mixes
     double m[8];        // matrix entries (U1: 2x2, D2 and PH: phases); OP_U2 and OP_DG read the gate's own
 };
 
@@ -548,7 +554,8 @@ int phase_kind(const double *e)
     return PHASE_ANY;
 }
 
-void classify(int n, const hq_gate &g, Item &it)
+// max_block: the widest dense gate that a pass of blocks may take (2: none)
+void classify(int n, const hq_gate &g, int max_block, Item &it)
 {
     const int k = g.k, K = 1 << k;
     const double *m = g.matrix;
@@ -589,7 +596,10 @@ void classify(int n, const hq_gate &g, Item &it)
         return;
     }
     if (k > 2) {
-        it.wide = true;
+        it.kind = OP_BLK;
+        it.wide = k > max_block;
+        it.pool = 0;
+        it.need = it.all | kNever;
         return;
     }
     // k = 2: a controlled gate, an exchange with phases, or dense.  Entries within 4 FP64 epsilon of the largest
@@ -689,24 +699,33 @@ struct Budget {
     }
 };
 
+// What a gate asks of the tile: the bits it mixes (K = 0: register runs), or all of its bits (dense blocks of K
+// qubits).
+uint64_t need_of(const Item &i, int K)
+{
+    if (!K) return i.need;
+    return i.nb <= K ? i.all : i.all | kNever;
+}
+
 // Runs every gate that can run with the tile bits T, starting from the bits in
-// `from`; returns the points gained (3 per gate of two mixed bits, 1 otherwise)
-// and appends the gates to out when given.
-int absorb(const Queues &q, int *head, uint64_t T, uint64_t from, Budget &bud, std::vector<int> *out)
+// `from`; returns the points gained (3 per gate of two or more needed bits, 1
+// otherwise) and appends the gates to out when given.
+int absorb(const Queues &q, int *head, uint64_t T, uint64_t from, int K, Budget &bud, std::vector<int> *out)
 {
     int points = 0;
     while (from) {
         const int b = __builtin_ctzll(from);
         const int g = q.front(head, b);
-        if (g < 0 || (q.it[g].need & ~T) || !bud.fits(q.it[g]) || !q.ready(head, g)) {
+        if (g < 0 || (need_of(q.it[g], K) & ~T) || !bud.fits(q.it[g]) || !q.ready(head, g)) {
             from &= from - 1;
             continue;
         }
         const Item &i = q.it[g];
         for (int j = 0; j < i.nb; ++j) ++head[i.bit[j]];
         from |= i.all;
-        bud.add(i);
-        points += (i.need & (i.need - 1)) ? 3 : 1;
+        if (!K) bud.add(i);
+        const uint64_t need = need_of(i, K);
+        points += (need & (need - 1)) ? 3 : 1;
         if (out) out->push_back(g);
     }
     return points;
@@ -904,6 +923,25 @@ double own_cost(const Item &i)
     return i.kind == OP_U1 && i.nb == 2 ? 0.55 : 1.0;
 }
 
+// Time of a gate in register runs and of a dense block in a block pass, ms at n = 28 (from whole circuits of 785 gates:
+// in runs 66.5 with CZ and 87 with fSim, in 139 three-qubit blocks 54.7, in 77 four-qubit blocks 59; QFT in runs); a
+// pass cannot take less than its read and write of the state.
+double run_cost(const Item &i)
+{
+    switch (i.kind) {
+    case OP_PH: return 0.05;
+    case OP_D2: return 0.13;
+    case OP_U2: return 0.22;
+    case OP_BLK: return i.nb == 3 ? 0.39 : 0.77;
+    default: return 0.10;
+    }
+}
+double block_cost(int K) { return K == 3 ? 0.39 : 0.77; }
+constexpr double kPassFloor = 0.75;
+// Below this size lists without 3- or 4-qubit gates stay on register runs (depth-12 CZ circuits, runs / blocks: n=25
+// 4.88 / 3.99 ms, n=23 1.28 / 1.20 ms; below, the plan of the blocks and their products cost the host more than that).
+constexpr int kBlockMinQubits = 23;
+
 // Tile bits and the length of its contiguous runs.  A larger tile takes more gates per pass; a smaller one gives
 // the SMs more tiles of a small state (and complex128, bound by the two FP64 lanes of an SM, wants all SMs).
 // Measured, us per random grid circuit (tile / run bits):
@@ -923,57 +961,91 @@ template <typename R> void tile_shape(int n, int &L, int &cmin)
 }
 
 // The gates [g0, g1) of the list, none of them wide, pass by pass.
+enum PassKind { PASS_RUNS, PASS_BLOCKS, PASS_SINGLE };
 template <typename R> struct Segment {
     const std::vector<Item> &it;
     const hq_gate *gates;
     Queues q;
     int n, L, cmin, left;
+    int K = 0;              // width of dense blocks, 0: none
     std::vector<int> list;  // the gates of the current pass, in a valid order
+    uint64_t T = 0;         // its tile (PASS_RUNS, PASS_BLOCKS)
 
     Segment(const std::vector<Item> &items, const hq_gate *gs, int n_, int g0, int g1)
         : it(items), gates(gs), q(items, n_, g0, g1), n(n_), left(g1 - g0)
     {
         tile_shape<R>(n, L, cmin);
+        if (sizeof(R) == 4 && L >= kBlockTileMin) {
+            if (n >= kBlockMinQubits) K = 3;
+            for (int g = g0; g < g1; ++g)
+                if (it[size_t(g)].kind == OP_BLK) K = std::max<int>(K, it[size_t(g)].nb);
+        }
     }
 
-    // The next pass into p; single is set instead when its gates (list) are cheaper on their own kernels.
-    void next(PassParam<R> &p, bool &single)
+    // The tile's bits and the gates of a pass: the contiguous low bits, then, as long as there is room, the ones that
+    // let the most gates in per added bit.  kind: 0 for register runs, else the width of dense blocks.
+    void grow(int kind, int *head, std::vector<int> &out, uint64_t &tile)
     {
         const uint64_t every = (uint64_t(1) << n) - 1;
-        int saved[HQ_MAX_N];
-        std::memcpy(saved, q.head, sizeof(int) * size_t(n));
-        list.clear();
+        out.clear();
         Budget bud;
-        // the tile's bits: the contiguous low ones, then, as long as there is room, the ones that let the most
-        // gates in per added bit
-        uint64_t T = n == L ? every : (uint64_t(1) << cmin) - 1;
-        absorb(q, q.head, T, every, bud, &list);
-        while (__builtin_popcountll(T) < L) {
-            const int room = L - __builtin_popcountll(T);
+        tile = n == L ? every : (uint64_t(1) << cmin) - 1;
+        absorb(q, head, tile, every, kind, bud, &out);
+        while (__builtin_popcountll(tile) < L) {
+            const int room = L - __builtin_popcountll(tile);
             uint64_t best = 0;
             double top = 0;
             for (int b = 0; b < n; ++b) {
-                const int g = q.front(q.head, b);
+                const int g = q.front(head, b);
                 if (g < 0) continue;
-                const uint64_t add = it[size_t(g)].need & ~T;
-                if (!add || __builtin_ctzll(it[size_t(g)].need & ~T) != b || __builtin_popcountll(add) > room ||
-                    !q.ready(q.head, g))
+                const uint64_t add = need_of(it[size_t(g)], kind) & ~tile;
+                if (!add || (add & kNever) || __builtin_ctzll(add) != b || __builtin_popcountll(add) > room ||
+                    !q.ready(head, g))
                     continue;
                 int h[HQ_MAX_N];
-                std::memcpy(h, q.head, sizeof(int) * size_t(n));
+                std::memcpy(h, head, sizeof(int) * size_t(n));
                 Budget b2 = bud;
-                const double gain = double(absorb(q, h, T | add, add, b2, nullptr)) / __builtin_popcountll(add);
+                const double gain =
+                    double(absorb(q, h, tile | add, add, kind, b2, nullptr)) / __builtin_popcountll(add);
                 if (gain > top) top = gain, best = add;
             }
             if (!best) break;
-            T |= best;
-            absorb(q, q.head, T, best, bud, &list);
+            tile |= best;
+            absorb(q, head, tile, best, kind, bud, &out);
         }
-        for (int b = 0; b < n && __builtin_popcountll(T) < L; ++b) T |= uint64_t(1) << b;
+        for (int b = 0; b < n && __builtin_popcountll(tile) < L; ++b) tile |= uint64_t(1) << b;
+    }
+
+    // The next pass: register runs (into p), dense blocks (list and T), or single gates cheaper on their own kernels.
+    PassKind next(PassParam<R> &p)
+    {
+        int saved[HQ_MAX_N];
+        std::memcpy(saved, q.head, sizeof(int) * size_t(n));
+        grow(0, q.head, list, T);
+        PassKind kind = PASS_RUNS;
+        if (K) {
+            // the kind that does more work per time (work: what the gates cost in register runs)
+            int head[HQ_MAX_N];
+            std::memcpy(head, saved, sizeof(int) * size_t(n));
+            std::vector<int> blist;
+            uint64_t btile = 0;
+            grow(K, head, blist, btile);
+            double runs = 0, work = 0;
+            for (int g : list) runs += run_cost(it[size_t(g)]);
+            for (int g : blist) work += run_cost(it[size_t(g)]);
+            const double rate = list.empty() ? 0.0 : runs / std::max(kPassFloor, runs);
+            if (!blist.empty() &&
+                work / std::max(kPassFloor, block_cost(K) * count_in_tile(n, K, gates, blist)) > rate) {
+                kind = PASS_BLOCKS;
+                list.swap(blist);
+                T = btile;
+                std::memcpy(q.head, head, sizeof(int) * size_t(n));
+            }
+        }
         double own = 0;
         for (int g : list) own += own_cost(it[size_t(g)]);
-        single = list.size() == 1 || (n >= 24 && own <= 1.0);
-        while (!single && !compile_pass<R>(p, n, L, T, it, gates, list)) {
+        if (list.size() == 1 || (n >= 24 && own <= 1.0)) kind = PASS_SINGLE;
+        while (kind == PASS_RUNS && !compile_pass<R>(p, n, L, T, it, gates, list)) {
             // too many runs: a shorter pass (the first half of the list is a valid order of its own)
             list.resize(list.size() / 2);
             std::memcpy(q.head, saved, sizeof(int) * size_t(n));
@@ -981,6 +1053,7 @@ template <typename R> struct Segment {
                 for (int j = 0; j < it[size_t(g)].nb; ++j) ++q.head[it[size_t(g)].bit[j]];
         }
         left -= int(list.size());
+        return kind;
     }
 };
 
@@ -992,22 +1065,28 @@ hq_status run_segment(void *state, int n, const std::vector<Item> &it, const hq_
     const hq_dtype dt = sizeof(R) == 4 ? HQ_C64 : HQ_C128;
     Segment<R> seg(it, gates, n, g0, g1);
     PassParam<R> p;
+    std::vector<TileBlock> blocks;
     while (seg.left > 0) {
-        bool single = false;
-        seg.next(p, single);
-        if (single) {
-            for (int g : seg.list) {
-                hq_status st = launch_gate(state, n, dt, gates[g].k, gates[g].qubits, gates[g].matrix, 1, engine, s);
-                if (st != HQ_OK) return st;
-            }
-            continue;
+        hq_status st = HQ_OK;
+        switch (seg.next(p)) {
+        case PASS_SINGLE:
+            for (int g : seg.list)
+                if ((st = launch_gate(state, n, dt, gates[g].k, gates[g].qubits, gates[g].matrix, 1, engine, s)) != HQ_OK)
+                    return st;
+            break;
+        case PASS_BLOCKS:
+            fuse_in_tile(n, seg.K, seg.T, gates, seg.list, blocks);
+            st = launch_block_pass(state, n, seg.L, seg.T, seg.K, blocks, s);
+            break;
+        default: {
+            const size_t smem = pass_smem<R>(p.L);
+            const int threads = std::max(32, std::min(kRunThreads, 1 << (p.L - Traits<R>::RP)));
+            const void *fn = (const void *)k_runs<R>;
+            const int grid = grid_for(fn, kRunThreads, smem, int64_t(1) << (n - p.L));
+            k_runs<R><<<grid, threads, smem, s>>>(p, (T2 *)state);
+            st = cuda_status("k_runs", cudaGetLastError());
         }
-        const size_t smem = pass_smem<R>(p.L);
-        const int threads = std::max(32, std::min(kRunThreads, 1 << (p.L - Traits<R>::RP)));
-        const void *fn = (const void *)k_runs<R>;
-        const int grid = grid_for(fn, kRunThreads, smem, int64_t(1) << (n - p.L));
-        k_runs<R><<<grid, threads, smem, s>>>(p, (T2 *)state);
-        hq_status st = cuda_status("k_runs", cudaGetLastError());
+        }
         if (st != HQ_OK) return st;
     }
     return HQ_OK;
@@ -1025,7 +1104,10 @@ hq_status run_list(void *state, int n, const hq_gate *gates, int G, int engine, 
         const int cnt = std::min(kMaxSegment, G - first);
         const hq_gate *const gs = gates + first;
         it.resize(size_t(cnt));
-        for (int g = 0; g < cnt; ++g) classify(n, gs[g], it[size_t(g)]);
+        int L = 0, c = 0;
+        tile_shape<R>(n, L, c);
+        const int max_block = sizeof(R) == 4 && L >= kBlockTileMin ? 4 : 2;
+        for (int g = 0; g < cnt; ++g) classify(n, gs[g], max_block, it[size_t(g)]);
         for (int g = 0; g < cnt;) {
             int e = g;
             while (e < cnt && !it[size_t(e)].wide) ++e;

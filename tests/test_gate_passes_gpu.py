@@ -90,6 +90,27 @@ def test_lists_match_oracle_and_single_gates(hq, n, count, wide, dt):
             assert float(torch.linalg.norm(d)) <= 2e-5 * max(1.0, count / 1000)
 
 
+@pytest.mark.parametrize("n", [9, 10, 11, 12, 13, 14, 18, 19, 23])
+@pytest.mark.parametrize("kmax", [3, 4])
+def test_dense_blocks_in_passes(hq, n, kmax):
+    """Lists of dense 3- and 4-qubit blocks (complex64: several per pass over the state) with narrow, diagonal and
+    wider gates between them, blocks on the lowest and highest bits, more blocks than one launch takes."""
+    sm, rng = C.SplitMix64(n + kmax), np.random.default_rng(n)
+    gates = gate_list(n, 20, n, True)
+    for _ in range(24):
+        k = int(rng.integers(2, kmax + 1))
+        qs = rng.choice(n, k, replace=False) if rng.uniform() < 0.7 else rng.permutation(n - k + np.arange(k))
+        gates.append(C.Gate("U", tuple(int(q) for q in qs), C.random_unitary(k, sm)))
+        if rng.uniform() < 0.2:
+            gates += gate_list(n, 2, int(rng.integers(1000)), False)
+    gates.insert(30, C.Gate("U5", (0, n - 1, 3, 1, n - 2), C.random_unitary(5, sm)))
+    psi = oracle.state_init(n, "+-" * (n // 2) + "1" * (n % 2))
+    st = torch.from_numpy(psi).to(torch.complex64).cuda()
+    hq.hq_apply_blocks(st, gates)
+    want = oracle.apply_circuit(psi.copy(), C.Circuit(n, gates))
+    assert np.linalg.norm(st.cpu().numpy() - want) <= 2e-5  # the stated tolerance up to 1000 gates
+
+
 @pytest.mark.parametrize("n", [12, 27])
 def test_qft_list(hq, n):
     """Hundreds of controlled phases between the Hadamards: QFT of a basis state is a plane wave."""
