@@ -153,7 +153,7 @@ __device__ __forceinline__ double flip(double w, int odd)
 // mask, the weights of a run summed first (an FP64 instruction costs 64 cycles
 // of an SM quarter; weights once per BC sets instead of products per set).
 // With a load, a popcount and a complex multiply-add per term and state, n = 20, 39 terms: batch 64 complex64 4.43
-// ms, batch 16 complex128 7.12 ms, against 1 GB / 0.5 GB of traffic; this: HAM64 and 2.68 ms.
+// ms, batch 16 complex128 7.12 ms, against 1 GB / 0.5 GB of traffic; this: 1.66 and 2.68 ms.
 template <typename R, int BC>
 __global__ void __launch_bounds__(kAdjThreads) k_ham(const __grid_constant__ HamParams p,
                                                      const typename C2<R>::type *__restrict__ phi,
@@ -173,7 +173,19 @@ __global__ void __launch_bounds__(kAdjThreads) k_ham(const __grid_constant__ Ham
         T2 out[BC];
 #pragma unroll
         for (int b = 0; b < BC; ++b) out[b].x = out[b].y = 0;
-        for (int t = 0; t < p.T;) {
+        if constexpr (BC == 1) {  // one set: loads of several terms in flight
+#pragma unroll 4
+            for (int t = 0; t < p.T; ++t) {
+                const HamTerm &h = p.t[t];
+                const T2 a = sp[x ^ int64_t(h.xm)];
+                const int odd = __popcll(uint64_t(x) & h.zm) & 1;
+                T2 w;
+                w.x = flip(sizeof(R) == 4 ? R(h.wrf) : R(h.wr), odd);
+                w.y = flip(sizeof(R) == 4 ? R(h.wif) : R(h.wi), odd);
+                cmac(out[0], w, a);
+            }
+        }
+        for (int t = 0; BC > 1 && t < p.T;) {
             const T2 *const from = sp + (x ^ int64_t(p.t[t].xm));
             bool last = false;
             if constexpr (sizeof(R) == 4) {
