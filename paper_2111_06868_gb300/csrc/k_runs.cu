@@ -31,7 +31,7 @@
 // From 23 qubits on (and for 3- and 4-qubit gates) a complex64 pass may instead fuse its gates into dense blocks
 // (k_block_pass.cu); the kind that does more work per time is chosen pass by pass.
 // Per-gate circuits, against one launch per gate: n=28 complex64 depth 20 fSim 528 -> 87 ms (55 in blocks), n=20
-// depth 16 CZ 1.53 -> 0.25 ms of device time, n=12 complex128 depth 10 1.06 -> 0.24 ms.
+// depth 16 CZ 1.53 -> 0.25 ms of device time, n=12 complex128 depth 10 1.06 -> 0.20 ms.
 #include <algorithm>
 #include <cmath>
 #include <cstring>
@@ -204,12 +204,12 @@ __device__ __forceinline__ double2 times_iy(const double2 m, double2 v)
     return m.y > 0 ? make_double2(-v.y, v.x) : make_double2(v.y, -v.x);
 }
 
-template <typename R, int P, int CLS>
-__device__ __forceinline__ void op_u1_class(typename Amp<R>::type (&a)[1 << Traits<R>::RP],
+template <typename R, int P, int CLS, int NA>
+__device__ __forceinline__ void op_u1_class(typename Amp<R>::type (&a)[NA],
                                       const typename Amp<R>::entry *m)
 {
     using T2 = typename Amp<R>::type;
-    constexpr int NA = 1 << Traits<R>::RP, H = NA / 2;
+    constexpr int H = NA / 2;
     constexpr int STEP = H < 4 ? H : 4;  // pairs per batch
     constexpr bool DI = CLS == U1_FULL || sizeof(R) == 8, OR = CLS != U1_REAL_IMAG || sizeof(R) == 8, OI = CLS != U1_REAL || sizeof(R) == 8;
     const auto m00 = m[0], m01 = m[1], m10 = m[2], m11 = m[3];
@@ -243,12 +243,12 @@ template <int P, int Q> __device__ __forceinline__ constexpr int pair_base(int g
     return ((x >> Q) << (Q + 1)) | (x & ((1 << Q) - 1));
 }
 
-template <typename R, int P, int Q>
-__device__ __forceinline__ void op_u2(typename Amp<R>::type (&a)[1 << Traits<R>::RP],
+template <typename R, int P, int Q, int NA>
+__device__ __forceinline__ void op_u2(typename Amp<R>::type (&a)[NA],
                                       const typename Amp<R>::entry *m)
 {
     using T2 = typename Amp<R>::type;
-    constexpr int NG = (1 << Traits<R>::RP) / 4, STEP = 2;
+    constexpr int NG = NA / 4, STEP = NG < 2 ? NG : 2;
 #pragma unroll
     for (int b = 0; b < NG; b += STEP) {
         T2 v[4][STEP], o[4][STEP];
@@ -271,11 +271,11 @@ __device__ __forceinline__ void op_u2(typename Amp<R>::type (&a)[1 << Traits<R>:
 }
 
 // entry r of m on the amplitudes whose bits Q, P are r; kinds: 4 bits per entry (PhaseKind)
-template <typename R, int P, int Q>
-__device__ __forceinline__ void op_d2(typename Amp<R>::type (&a)[1 << Traits<R>::RP],
+template <typename R, int P, int Q, int NA>
+__device__ __forceinline__ void op_d2(typename Amp<R>::type (&a)[NA],
                                       const typename Amp<R>::entry *m, int kinds)
 {
-    constexpr int NG = (1 << Traits<R>::RP) / 4;
+    constexpr int NG = NA / 4;
 #pragma unroll
     for (int r = 0; r < 4; ++r) {
         const int kind = (kinds >> (4 * r)) & 15;
@@ -298,11 +298,10 @@ __device__ __forceinline__ void op_d2(typename Amp<R>::type (&a)[1 << Traits<R>:
 }
 
 // a phase on the amplitudes whose register bits MASK are all 1
-template <typename R, int MASK>
-__device__ __forceinline__ void op_ph(typename Amp<R>::type (&a)[1 << Traits<R>::RP],
+template <typename R, int MASK, int NA>
+__device__ __forceinline__ void op_ph(typename Amp<R>::type (&a)[NA],
                                       const typename Amp<R>::entry d, bool minus)
 {
-    constexpr int NA = 1 << Traits<R>::RP;
     if (minus) {
 #pragma unroll
         for (int j = 0; j < NA; ++j)
@@ -317,14 +316,14 @@ __device__ __forceinline__ void op_ph(typename Amp<R>::type (&a)[1 << Traits<R>:
 // one gate body per case; Q: the highest register position it uses
 #define HQ_CASE(Q, CODE, ...)                             \
     case CODE:                                            \
-        if constexpr ((Q) < Traits<R>::RP) __VA_ARGS__;   \
+        if constexpr ((Q) < RP) __VA_ARGS__;              \
         break
 
-template <typename R>
-__device__ __forceinline__ void apply_op(const RunOp &op, typename Amp<R>::type (&a)[1 << Traits<R>::RP], int i0,
+template <typename R, int RP>
+__device__ __forceinline__ void apply_op(const RunOp &op, typename Amp<R>::type (&a)[1 << RP], int i0,
                                          uint64_t base, const typename Amp<R>::entry *pool, const uint8_t *aux)
 {
-    constexpr int RP = Traits<R>::RP, NA = 1 << RP;
+    constexpr int NA = 1 << RP;
     const auto *m = reinterpret_cast<const typename Amp<R>::entry *>(reinterpret_cast<const char *>(pool) + op.mat);
     if (op.var && ((i0 & op.lmask) != op.lmask || (base & op.omask) != op.omask)) return;  // a control is 0
     switch (op.code) {
@@ -396,14 +395,14 @@ template <typename R> constexpr size_t pass_smem(int L)
            sizeof(RunDesc) * kMaxRuns + sizeof(RunOp) * (kMaxOps + 1) + kMaxAux;
 }
 
-template <typename R>
+template <typename R, int RP>
 __global__ void __launch_bounds__(kRunThreads, 3) k_runs(const __grid_constant__ PassParam<R> p,
                                                          typename C2<R>::type *__restrict__ state)
 {
     using T2 = typename C2<R>::type;
     using A = typename Amp<R>::type;
     using PE = typename Amp<R>::entry;
-    constexpr int RP = Traits<R>::RP, NA = 1 << RP, NB = Traits<R>::NB;
+    constexpr int NA = 1 << RP, NB = Traits<R>::NB;
     constexpr int V = 16 / int(sizeof(T2));  // amplitudes per 16-byte copy
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int L = p.L, c = p.c, nh = L - c;
@@ -483,7 +482,7 @@ __global__ void __launch_bounds__(kRunThreads, 3) k_runs(const __grid_constant__
 #pragma unroll 1
                 for (int o = op0; o < op1; ++o) {
                     const RunOp next = ops[o + 1];  // in flight under this gate (slot kMaxOps exists)
-                    apply_op<R>(op, a, i0, uint64_t(base), pool, aux);
+                    apply_op<R, RP>(op, a, i0, uint64_t(base), pool, aux);
                     op = next;
                 }
                 {
@@ -742,11 +741,11 @@ void put_entry(PassParam<R> &p, int at, const double *e)
 // kernel's parameters.  T: the tile's flat bits (L of them, the lowest c
 // contiguous).  False when the runs do not fit (the caller then shortens the
 // list).
-template <typename R>
+template <typename R, int RP>
 bool compile_pass(PassParam<R> &p, int n, int L, uint64_t T, const std::vector<Item> &it, const hq_gate *gates,
                   std::vector<int> list)
 {
-    constexpr int RP = Traits<R>::RP, NB = Traits<R>::NB, NA = 1 << RP;
+    constexpr int NB = Traits<R>::NB, NA = 1 << RP;
     p.n = n;
     p.L = L;
     int c = 0;
@@ -948,21 +947,26 @@ constexpr int kBlockMinQubits = 23;
 //   complex64   n=12  12/5 56   11/4 54   9/4 60      n=18  13/5 231  12/4 138  11/4 120  10/4 133
 //               n=20  13/5 309  12/4 246  11/4 306    n=22  13/5 771  12/4 672  11/4 885
 //               n=24  13/5 2730 13/6 2853 12/4 2849   n=26  13/5 10047  12/4 10282  11/4 13533
-//   complex128  n=12  12/4 817  10/4 254  9/3 239  8/3 245   n=16  10/4 430  9/3 404  8/2 410
+//   complex128  n=12  10/4 350  9/3 209  8/3 197  7/3 216    n=16  10/4 577  9/3 354  8/3 349  (4 amplitudes per thread)
 //               n=18  12/4 1755  11/4 922  10/4 928  9/3 1193
 //               n=20  11/4 2723  10/4 2449  9/3 2670         n=23  12/4 21449  11/4 20833  10/4 21338
 template <typename R> void tile_shape(int n, int &L, int &cmin)
 {
     if (sizeof(R) == 4) L = n >= 23 ? 13 : n >= 19 ? 12 : 11;
-    else L = n >= 21 ? 11 : n >= 17 ? 10 : 9;
-    cmin = L == 13 ? 5 : L == 9 ? 3 : 4;
+    else L = n >= 21 ? 11 : n >= 17 ? 10 : 8;
+    cmin = L == 13 ? 5 : L == 8 ? 3 : 4;
     L = std::min(L, n);
     cmin = std::min(cmin, L);
 }
 
+// Up to this size complex128 passes take 4 amplitudes per thread instead of 8: an FP64 instruction takes a quarter of an
+// SM 64 cycles whatever its lanes do, so a small state wants its gates on as many warps as it can fill (4 / 8: n=12 197
+// / 238 us, n=16 349 / 404; n=18 1427 / 927).
+constexpr int kFewQubits128 = 16;
+
 // The gates [g0, g1) of the list, none of them wide, pass by pass.
 enum PassKind { PASS_RUNS, PASS_BLOCKS, PASS_SINGLE };
-template <typename R> struct Segment {
+template <typename R, int RP> struct Segment {
     const std::vector<Item> &it;
     const hq_gate *gates;
     Queues q;
@@ -1045,7 +1049,7 @@ template <typename R> struct Segment {
         double own = 0;
         for (int g : list) own += own_cost(it[size_t(g)]);
         if (list.size() == 1 || (n >= 24 && own <= 1.0)) kind = PASS_SINGLE;
-        while (kind == PASS_RUNS && !compile_pass<R>(p, n, L, T, it, gates, list)) {
+        while (kind == PASS_RUNS && !compile_pass<R, RP>(p, n, L, T, it, gates, list)) {
             // too many runs: a shorter pass (the first half of the list is a valid order of its own)
             list.resize(list.size() / 2);
             std::memcpy(q.head, saved, sizeof(int) * size_t(n));
@@ -1057,13 +1061,13 @@ template <typename R> struct Segment {
     }
 };
 
-template <typename R>
+template <typename R, int RP>
 hq_status run_segment(void *state, int n, const std::vector<Item> &it, const hq_gate *gates, int g0, int g1,
                       int engine, cudaStream_t s)
 {
     using T2 = typename C2<R>::type;
     const hq_dtype dt = sizeof(R) == 4 ? HQ_C64 : HQ_C128;
-    Segment<R> seg(it, gates, n, g0, g1);
+    Segment<R, RP> seg(it, gates, n, g0, g1);
     PassParam<R> p;
     std::vector<TileBlock> blocks;
     while (seg.left > 0) {
@@ -1080,10 +1084,10 @@ hq_status run_segment(void *state, int n, const std::vector<Item> &it, const hq_
             break;
         default: {
             const size_t smem = pass_smem<R>(p.L);
-            const int threads = std::max(32, std::min(kRunThreads, 1 << (p.L - Traits<R>::RP)));
-            const void *fn = (const void *)k_runs<R>;
+            const int threads = std::max(32, std::min(kRunThreads, 1 << (p.L - RP)));
+            const void *fn = (const void *)k_runs<R, RP>;
             const int grid = grid_for(fn, kRunThreads, smem, int64_t(1) << (n - p.L));
-            k_runs<R><<<grid, threads, smem, s>>>(p, (T2 *)state);
+            k_runs<R, RP><<<grid, threads, smem, s>>>(p, (T2 *)state);
             st = cuda_status("k_runs", cudaGetLastError());
         }
         }
@@ -1113,7 +1117,9 @@ hq_status run_list(void *state, int n, const hq_gate *gates, int G, int engine, 
             while (e < cnt && !it[size_t(e)].wide) ++e;
             hq_status st = HQ_OK;
             if (e - g > 1) {
-                st = run_segment<R>(state, n, it, gs, g, e, engine, s);
+                constexpr int RP = Traits<R>::RP, FEW = sizeof(R) == 8 ? 2 : RP;
+                st = n <= kFewQubits128 ? run_segment<R, FEW>(state, n, it, gs, g, e, engine, s)
+                                        : run_segment<R, RP>(state, n, it, gs, g, e, engine, s);
             } else {
                 e = g + 1;
                 st = launch_gate(state, n, dt, gs[g].k, gs[g].qubits, gs[g].matrix, 1, engine, s);
