@@ -60,7 +60,7 @@ __device__ __forceinline__ unsigned long long b_fma(unsigned long long x, unsign
 }
 
 template <int K, int NB>
-__global__ void __launch_bounds__(kBpThreads, K == 3 ? 3 : 2) k_block_pass(const __grid_constant__ BlockPassParam<K, NB> p,
+__global__ void __launch_bounds__(kBpThreads, 3) k_block_pass(const __grid_constant__ BlockPassParam<K, NB> p,
                                                                           float2 *__restrict__ state)
 {
     constexpr int D = 1 << K;
