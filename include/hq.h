@@ -252,8 +252,9 @@ typedef struct {
  *   u:      one uniform in [0, 1) per channel, in operation order.
  *   chosen: out (may be NULL), the sampled Kraus index per channel.
  * Channels whose operators all have K_i^dag K_i = p_i I are sampled on the
- * host from p_i alone; the others on the device (reduced density matrix,
- * branch and renormalised operator picked by one CTA, no host round trip).
+ * host from p_i alone; the others on the device, no host round trip (n >= 4:
+ * two one-qubit channels on different qubits at a time, from their joint reduced
+ * density matrix, when nothing but folded operators lies between them).
  * The operators applied right before a device-sampled channel on the same
  * qubits, in the same order, are folded into it (probabilities from
  * A rho A^dag, K_i A / sqrt(p_i) applied): the same result in fewer passes.

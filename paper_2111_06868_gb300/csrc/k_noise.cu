@@ -5,10 +5,12 @@
 //     the other qubits, in one read of the state.  Pure-state sampling of a
 //     Kraus channel (Sec. 5) takes its branch probabilities from it:
 //     p_i = ||K_i psi||^2 = Tr(K_i rho K_i^dag).
-//   * k_kraus_pick, k_apply_sel: the branch of a state-dependent channel
-//     picked on the device from k_rdm's partial sums and a caller-drawn
-//     uniform, and the renormalised Kraus operator applied, with no host
-//     round trip.
+//   * k_window (n >= 4): one or two state-dependent channels per pass: the
+//     branches picked on the device from the partial sums of the launch before
+//     and caller-drawn uniforms, the renormalised operators applied, the next
+//     window's reduced density matrix summed from what is written.
+//   * k_kraus_pick, k_apply_sel (n < 4): the same channel by channel from
+//     k_rdm's partial sums.
 // Each thread sums its share of a complex64 state in FP32 with a compensation
 // term (complex128 in FP64), the CTA sums in FP64; one CTA joins the CTAs'
 // sums in a fixed order.  At most two CTAs per SM, so that few partial
@@ -442,8 +444,10 @@ static hq_status sample_on_device(void *state, int n, const int *qubits, PickArg
 // write of the state instead of a read, a one-CTA pick and a read and write.
 // A thread holds 16 amplitudes: all values of this window's two qubits and of
 // the next one's (a qubit that a window lacks is replaced by any other bit).
-// Bound: HBM (two channels at n = 24: 268 MB, 40 us at the copy bandwidth), with
-// about 5 us of FP64 latency per launch for the pick; complex128 the FP64 pipe.
+// Bound: HBM (two channels at n = 24: 268 MB, 40 us at the copy bandwidth; the
+// launch takes 67-73 us with cold caches, where three launches per channel took
+// 101), with about 5 us of FP64 latency per launch for the pick; complex128 the
+// FP64 pipe.
 // ----------------------------------------------------------------------------
 constexpr int kWindowRow = 20;  // sums per CTA: 10 complex entries of the upper triangle
 struct WindowParam {
