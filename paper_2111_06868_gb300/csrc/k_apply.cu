@@ -523,6 +523,7 @@ __device__ __forceinline__ float2 pair_split(unsigned long long v)
 }
 
 constexpr int kPairTileBits = 11, kPairThreads = 128;
+constexpr int kPairMinQubits = 20;  // K = 4
 
 template <int K>
 __global__ void __launch_bounds__(kPairThreads, 4) k_gather_pair(const __grid_constant__ TileGeom g,
@@ -560,12 +561,64 @@ __global__ void __launch_bounds__(kPairThreads, 4) k_gather_pair(const __grid_co
     else tiles_pipelined_lean<kPairTileBits, kPairThreads>(g, state, op);
 }
 
-// K = 1, 2 in complex64: bound by HBM with plain FMAs
+// K = 4 in complex64 on fewer than kPairMinQubits qubits: four threads per
+// group (a small state has few groups, and one thread's 16 rows are a long
+// chain: n = 10, ten blocks 45 against 56 us), as gather_tile's chunked form, with the matrix read
+// from shared memory (every lane of a warp reads the same entry: a
+// broadcast) at a row offset known only at run time, so that one copy of the
+// unrolled 4 x 16 multiply-add body serves all four row chunks (four
+// constant-operand copies of it did not stay in the instruction cache).
+// (Packed FMAs with the entries stored as (Re, Re, -Im, Im) took 20 % longer:
+// one 16-byte shared load per complex multiply-add.)
+template <int LB>
+__device__ __forceinline__ void gather_tile_k4_sh(const TileGeom &g, const float2 (*msh)[16], float2 *tile)
+{
+    constexpr int K = 4, NR = gather_rows<float, K>(), TPG = gather_tpg<float, K>(), NI = gather_items<float, K, LB>();
+    const int ngroups = (1 << g.L) >> K;
+    float2 acc[NI][NR];
+    int ibs[NI], chunk[NI];
+#pragma unroll
+    for (int it = 0; it < NI; ++it) {
+        const int w = it * kThreads + threadIdx.x;
+        const int wi = w >> 5;
+        chunk[it] = wi % TPG;
+        const int grp = (wi / TPG) * 32 + (w & 31);
+        ibs[it] = -1;
+#pragma unroll
+        for (int rr = 0; rr < NR; ++rr) acc[it][rr].x = acc[it][rr].y = 0;
+        if (grp < ngroups) {
+            ibs[it] = group_base<K>(g, grp);
+            const float2 (*mr)[16] = msh + chunk[it] * NR;
+#pragma unroll
+            for (int c = 0; c < (1 << K); ++c) {
+                const float2 v = tile[swz<float>(ibs[it] + g.toff[c])];
+#pragma unroll
+                for (int rr = 0; rr < NR; ++rr) cmac(acc[it][rr], mr[rr][c], v);
+            }
+        }
+    }
+    __syncthreads();
+#pragma unroll
+    for (int it = 0; it < NI; ++it)
+        if (ibs[it] >= 0)
+#pragma unroll
+            for (int rr = 0; rr < NR; ++rr) tile[swz<float>(ibs[it] + g.toff[chunk[it] * NR + rr])] = acc[it][rr];
+    __syncthreads();
+}
+
+// K = 1, 2 in complex64: bound by HBM with plain FMAs (K = 4: small states, above)
 template <int K>
 __global__ void __launch_bounds__(kThreads) k_gather_pipe(const TileGeom g, const MatParam<float, K> m,
                                                           float2 *__restrict__ state)
 {
-    tiles_pipelined(g, state, [&](float2 *tile) { gather_tile<float, K, 11>(g, m, tile); });
+    if constexpr (K == 4) {
+        __shared__ float2 msh[16][16];
+        for (int i = threadIdx.x; i < 256; i += blockDim.x) msh[i >> 4][i & 15] = m.a[i >> 4][i & 15];
+        // (tiles_pipelined's first barrier orders these stores before the reads)
+        tiles_pipelined(g, state, [&](float2 *tile) { gather_tile_k4_sh<11>(g, msh, tile); });
+    } else {
+        tiles_pipelined(g, state, [&](float2 *tile) { gather_tile<float, K, 11>(g, m, tile); });
+    }
 }
 
 // ----------------------------------------------------------------------------
@@ -907,35 +960,39 @@ static hq_status run_gather(void *state, int n, const int *qubits, const double 
         }
     // complex64: the next tile's load in flight under the current one (two buffers per CTA)
     if constexpr (sizeof(R) == 4 && K >= 3) {
-        make_geom(g, n, K, qubits, std::min(n, kPairTileBits), nstates);
-        PairMatParam<K> p;
-        for (int r = 0; r < (1 << K); ++r) {
-            p.off[r] = (g.toff[r] ^ ((g.toff[r] >> 4) & 15)) * int(sizeof(float2));
-            for (int c = 0; c < (1 << K); ++c) {
-                const float2 re = make_float2(m.a[r][c].x, m.a[r][c].x), im = make_float2(m.a[r][c].y, m.a[r][c].y);
-                std::memcpy(&p.a[r][c].x, &re, 8);
-                std::memcpy(&p.a[r][c].y, &im, 8);
+        if (K == 3 || n >= kPairMinQubits) {
+            make_geom(g, n, K, qubits, std::min(n, kPairTileBits), nstates);
+            PairMatParam<K> p;
+            for (int r = 0; r < (1 << K); ++r) {
+                p.off[r] = (g.toff[r] ^ ((g.toff[r] >> 4) & 15)) * int(sizeof(float2));
+                for (int c = 0; c < (1 << K); ++c) {
+                    const float2 re = make_float2(m.a[r][c].x, m.a[r][c].x), im = make_float2(m.a[r][c].y, m.a[r][c].y);
+                    std::memcpy(&p.a[r][c].x, &re, 8);
+                    std::memcpy(&p.a[r][c].y, &im, 8);
+                }
             }
+            const size_t smem = size_t(2 * sizeof(float2)) << g.L;
+            const void *fn = (const void *)k_gather_pair<K>;
+            const int grid = grid_for(fn, kPairThreads, smem, g.total_tiles);
+            k_gather_pair<K><<<grid, kPairThreads, smem, s>>>(g, p, (float2 *)state);
+            return cuda_status("k_gather_pair", cudaGetLastError());
         }
-        const size_t smem = size_t(2 * sizeof(float2)) << g.L;
-        const void *fn = (const void *)k_gather_pair<K>;
-        const int grid = grid_for(fn, kPairThreads, smem, g.total_tiles);
-        k_gather_pair<K><<<grid, kPairThreads, smem, s>>>(g, p, (float2 *)state);
-        return cuda_status("k_gather_pair", cudaGetLastError());
-    } else if constexpr (sizeof(R) == 4) {
+    }
+    if constexpr (sizeof(R) == 4 && K != 3) {
         make_geom(g, n, K, qubits, std::min(n, 11), nstates);
         const size_t smem = size_t(2 * sizeof(float2)) << g.L;
         const void *fn = (const void *)k_gather_pipe<K>;
         const int grid = grid_for(fn, kThreads, smem, g.total_tiles);
         k_gather_pipe<K><<<grid, kThreads, smem, s>>>(g, m, (float2 *)state);
         return cuda_status("k_gather_pipe", cudaGetLastError());
-    } else {
-    const size_t smem = size_t(sizeof(typename C2<R>::type)) << g.L;
-    const void *fn = (const void *)k_gather<R, K>;
-    const int grid = grid_for(fn, kThreads, smem, g.total_tiles);
-    k_gather<R, K><<<grid, kThreads, smem, s>>>(g, m, (typename C2<R>::type *)state);
-    return cuda_status("k_gather", cudaGetLastError());
+    } else if constexpr (sizeof(R) == 8) {
+        const size_t smem = size_t(sizeof(typename C2<R>::type)) << g.L;
+        const void *fn = (const void *)k_gather<R, K>;
+        const int grid = grid_for(fn, kThreads, smem, g.total_tiles);
+        k_gather<R, K><<<grid, kThreads, smem, s>>>(g, m, (typename C2<R>::type *)state);
+        return cuda_status("k_gather", cudaGetLastError());
     }
+    return HQ_OK;  // (not reached: complex64 K = 3 always takes k_gather_pair)
 }
 
 template <typename R, int K>

@@ -936,6 +936,34 @@ double run_cost(const Item &i)
     }
 }
 double block_cost(int K) { return K == 3 ? 0.39 : 0.77; }
+
+// complex128: the same for a gate in register runs and on its own kernel (ms at n = 28; FP64 multiply-adds at two per
+// clock and SM, 0.46 ms for one per amplitude; a read and write of the state 1.26 ms).  Measured at n = 22: a CNOT 43 us on
+// k_ctrl and 100 in runs (its 4 x 4 form tests every part), a dense two-qubit gate 154 and 157.
+double own_cost_128(const Item &i)
+{
+    switch (i.kind) {
+    case OP_PH: return i.nb == 1 ? 1.85 : 0.5;
+    case OP_U1: return i.nb == 2 ? 2.75 : 3.9;
+    case OP_U2: return 9.8;
+    default: return 1.9;
+    }
+}
+double run_cost_128(const Item &i)
+{
+    auto parts = [&](int n) {  // nonzero parts of the first n entries
+        int c = 0;
+        for (int e = 0; e < 2 * n; ++e) c += i.m[e] != 0.0;
+        return c;
+    };
+    switch (i.kind) {
+    case OP_PH: return i.flags ? 0.1 : 0.5;
+    case OP_U1: return i.nb == 2 ? 6.4 : 0.5 * parts(4);
+    case OP_U2: return 10.0;
+    case OP_D2: return 0.25 * parts(4);
+    default: return 2.0;
+    }
+}
 constexpr double kPassFloor = 0.75;
 // Below this size lists without 3- or 4-qubit gates stay on register runs (depth-12 CZ circuits, runs / blocks: n=25
 // 4.88 / 3.99 ms, n=23 1.28 / 1.20 ms; below, the plan of the blocks and their products cost the host more than that).
@@ -1046,9 +1074,18 @@ template <typename R, int RP> struct Segment {
                 std::memcpy(q.head, head, sizeof(int) * size_t(n));
             }
         }
-        double own = 0;
-        for (int g : list) own += own_cost(it[size_t(g)]);
-        if (list.size() == 1 || (n >= 24 && own <= 1.0)) kind = PASS_SINGLE;
+        double own = 0, own64 = 0, run64 = 0;
+        bool dense = false;
+        for (int g : list) {
+            const Item &i = it[size_t(g)];
+            own += own_cost(i);
+            dense = dense || i.kind == OP_U2;
+            if (sizeof(R) == 8) own64 += own_cost_128(i), run64 += run_cost_128(i);
+        }
+        if (list.size() == 1 || (n >= 20 && own <= 1.0)) kind = PASS_SINGLE;
+        // complex128: where the FP64 work of the gates is what counts, a pass saves nothing
+        if (sizeof(R) == 8 && (n >= 17 ? std::max(1.3, run64) >= 0.95 * own64 : list.size() <= 2 && dense))
+            kind = PASS_SINGLE;
         while (kind == PASS_RUNS && !compile_pass<R, RP>(p, n, L, T, it, gates, list)) {
             // too many runs: a shorter pass (the first half of the list is a valid order of its own)
             list.resize(list.size() / 2);
@@ -1110,7 +1147,8 @@ hq_status run_list(void *state, int n, const hq_gate *gates, int G, int engine, 
         it.resize(size_t(cnt));
         int L = 0, c = 0;
         tile_shape<R>(n, L, c);
-        const int max_block = sizeof(R) == 4 && L >= kBlockTileMin ? 4 : 2;
+        // (4-qubit blocks: below 20 qubits their own kernel is faster, n=18 115 against 123 us for 19 blocks)
+        const int max_block = sizeof(R) == 4 && L >= kBlockTileMin ? (n >= 20 ? 4 : 3) : 2;
         for (int g = 0; g < cnt; ++g) classify(n, gs[g], max_block, it[size_t(g)]);
         for (int g = 0; g < cnt;) {
             int e = g;
