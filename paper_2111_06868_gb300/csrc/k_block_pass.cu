@@ -20,6 +20,7 @@
 // 4-qubit blocks, n = 28: 64.1 ms one launch per block (k_gather_pair), 59.3 in passes; 3-qubit blocks n = 24: 3.72 -> 2.00
 // ms, n = 12: 213 -> 67 us.
 #include <algorithm>
+#include <cmath>
 #include <cstring>
 #include <vector>
 
@@ -188,6 +189,36 @@ void multiply_in(TileBlock &blk, int K, int n, const hq_gate &g)
     }
 }
 
+void identity_block(TileBlock &blk, int K, uint64_t qubits)
+{
+    const int D = 1 << K;
+    blk.k = 0;
+    for (uint64_t q = qubits; q; q &= q - 1) blk.bit[blk.k++] = __builtin_ctzll(q);
+    std::memset(blk.m, 0, sizeof(double) * size_t(2 * D * D));
+    for (int r = 0; r < D; ++r) blk.m[2 * (r * D + r)] = 1.0;
+}
+
+// Whether the product can stand in FP32 for its gates one after another: the
+// largest part of every column (that is not all zero) within 2^-64 .. 2^64.  Gates
+// far from unitary (scaled by 1e25, say) make products outside FP32's range
+// (overflow to infinity, flush to 0) although every state between them is inside.
+bool float_range(const TileBlock &blk, int K)
+{
+    const int D = 1 << K;
+    for (int c = 0; c < D; ++c) {
+        double mx = 0;
+        bool number = true;
+        for (int r = 0; r < D; ++r)
+            for (int x = 0; x < 2; ++x) {
+                const double v = std::fabs(blk.m[2 * (r * D + c) + x]);
+                number = number && v <= 0x1p64;  // (false for NaN)
+                mx = std::max(mx, v);
+            }
+        if (!number || (mx != 0.0 && mx < 0x1p-64)) return false;
+    }
+    return true;
+}
+
 template <int K, int NB>
 hq_status launch_blocks(void *state, int n, int L, uint64_t T, std::vector<TileBlock> &blocks, cudaStream_t s)
 {
@@ -272,19 +303,23 @@ void fuse_in_tile(int n, int K, uint64_t T, const hq_gate *gates, const std::vec
     std::vector<uint64_t> set;
     std::vector<int> member;
     group_in_tile(n, K, gates, list, set, member);
-    const int D = 1 << K;
     for (size_t b = 0; b < set.size(); ++b) {
         // a block of fewer qubits is widened by the tile's highest other bits (identity there)
         for (int x = 63; x >= 0 && __builtin_popcountll(set[b]) < K; --x)
             if (((T >> x) & 1) && !((set[b] >> x) & 1)) set[b] |= uint64_t(1) << x;
         blocks.emplace_back();
-        TileBlock &blk = blocks.back();
-        blk.k = 0;
-        for (uint64_t q = set[b]; q; q &= q - 1) blk.bit[blk.k++] = __builtin_ctzll(q);
-        std::memset(blk.m, 0, sizeof(double) * size_t(2 * D * D));
-        for (int r = 0; r < D; ++r) blk.m[2 * (r * D + r)] = 1.0;
+        identity_block(blocks.back(), K, set[b]);
         for (size_t i = 0; i < list.size(); ++i)
-            if (member[i] == int(b)) multiply_in(blk, K, n, gates[list[i]]);
+            if (member[i] == int(b)) multiply_in(blocks.back(), K, n, gates[list[i]]);
+        if (float_range(blocks.back(), K)) continue;
+        // the product leaves FP32's range where its gates need not: one block per gate
+        blocks.pop_back();
+        for (size_t i = 0; i < list.size(); ++i)
+            if (member[i] == int(b)) {
+                blocks.emplace_back();
+                identity_block(blocks.back(), K, set[b]);
+                multiply_in(blocks.back(), K, n, gates[list[i]]);
+            }
     }
 }
 
