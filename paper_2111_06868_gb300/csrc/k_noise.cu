@@ -12,9 +12,10 @@
 //   * k_kraus_pick, k_apply_sel (n < 4): the same channel by channel from
 //     k_rdm's partial sums.
 // Each thread sums its share of a complex64 state in FP32 with a compensation
-// term (complex128 in FP64), the CTA sums in FP64; one CTA joins the CTAs'
-// sums in a fixed order.  At most two CTAs per SM, so that few partial
-// sums reach that join.
+// term, 8 products per addition (complex128 in FP64).  k_rdm: the CTA sums in
+// FP64, one CTA joins the CTAs' sums; at most two CTAs per SM, so that few
+// partial sums reach that join.  k_window: see there; one CTA per SM.  All
+// joins run in a fixed order.
 #include <algorithm>
 #include <cmath>
 #include <cstring>
@@ -461,9 +462,9 @@ struct WindowParam {
     int nK[2];
     int *chosen[2];
     int *status;
-    const void *in;    // partial sums for this window: `rows` rows of kWindowRow Pair<R>
+    const double *in;  // partial sums for this window: `rows` rows of kWindowRow
     int rows;
-    void *out;         // partial sums for the next window, one row per CTA
+    double *out;       // partial sums for the next window, one row per CTA
 };
 
 // One warp: the branch of a channel on D levels with reduced density matrix
@@ -528,6 +529,8 @@ __device__ __forceinline__ bool window_pick(const double *rho0, const double *K,
     if (!(total > 0)) pick = -1;
     double mr = x == y ? 1.0 : 0.0, mi = 0;
     if (pick >= 0) {
+        // (rsqrt: at most 0.51 ulp off, 0.29 on average, over 2^23 values each in [2^-20, 1), [0.9, 1.1] and
+        // [2^-300, 2^300]; 1.0 / sqrt: 1.49 and 0.44 to 0.50)
         const double sc = rsqrt(ppick);
         const double *Kp = K + size_t(pick) * 2 * DD;
         mr = 0;
@@ -553,40 +556,66 @@ __device__ __forceinline__ bool window_pick(const double *rho0, const double *K,
     return identity;
 }
 
-// Sums of a window kernel: pairs (high, low) of the state's real type, joined by error-free additions (Knuth's
-// two-sum; the pair carries 48 bits for FP32).  An FP64 instruction takes a GB300 SM's quarter 64 cycles whatever its
-// lanes do: joined as doubles, the 20 sums of each of the 16 warps were 21 of a launch's 83 us.
-template <typename R> struct Pair {
-    R h, l;
+// Sums of a window kernel.  complex64: a thread hands over its compensated FP32 sum as a pair; inside the CTA the pairs
+// are joined in three-float sums (error-free additions, Knuth's two-sum: 70 bits and more, so no less than FP64's 53),
+// and the CTA's sums and those of all CTAs are FP64.  Joined as doubles from the threads on, the 20 sums of each of the
+// 16 warps were 21 of a launch's 83 us (an FP64 instruction takes a GB300 SM's quarter 64 cycles whatever its lanes do).
+template <typename R> struct ThreadSum;
+template <> struct ThreadSum<float> {
+    float h, l;
 };
-__device__ __forceinline__ Pair<float> pair_add(Pair<float> a, Pair<float> b)
-{
-    const float t = a.h + b.h, z = t - a.h;
-    const float e = ((a.h - (t - z)) + (b.h - z)) + (a.l + b.l);
-    Pair<float> r;
-    r.h = t + e;
-    r.l = e - (r.h - t);
-    return r;
-}
-__device__ __forceinline__ Pair<double> pair_add(Pair<double> a, Pair<double> b) { return {a.h + b.h, 0.0}; }
-// a thread's compensated sum
-__device__ __forceinline__ Pair<float> pair_of(float sum, float comp)
+template <> struct ThreadSum<double> {
+    double h;
+};
+__device__ __forceinline__ ThreadSum<float> thread_sum(float sum, float comp, float scale)
 {
     const float h = sum - comp;
-    return {h, (sum - h) - comp};
+    return {h * scale, ((sum - h) - comp) * scale};
 }
-__device__ __forceinline__ Pair<double> pair_of(double sum, double) { return {sum, 0.0}; }
+__device__ __forceinline__ ThreadSum<double> thread_sum(double sum, double, double) { return {sum}; }
+
+template <typename R> struct Sum;
+template <> struct Sum<float> {
+    float a, b, c;  // a + b + c, each about 2^-24 of the one before
+};
+template <> struct Sum<double> {
+    double a;
+};
+// x + y = result + err exactly
+__device__ __forceinline__ float two_sum(float x, float y, float &err)
+{
+    const float t = x + y, z = t - x;
+    err = (x - (t - z)) + (y - z);
+    return t;
+}
+__device__ __forceinline__ void sum_add(Sum<float> &s, float a, float b, float c)
+{
+    float d, e, g;
+    s.a = two_sum(s.a, a, d);
+    s.b = two_sum(s.b, d, e);
+    s.b = two_sum(s.b, b, g);
+    s.c += (e + g) + c;
+}
+__device__ __forceinline__ void sum_start(Sum<float> &s, ThreadSum<float> t) { s = {t.h, t.l, 0.f}; }
+__device__ __forceinline__ void sum_start(Sum<double> &s, ThreadSum<double> t) { s = {t.h}; }
+__device__ __forceinline__ void sum_add(Sum<float> &s, ThreadSum<float> t) { sum_add(s, t.h, t.l, 0.f); }
+__device__ __forceinline__ void sum_add(Sum<double> &s, ThreadSum<double> t) { s.a += t.h; }
+__device__ __forceinline__ double sum_value(Sum<float> s) { return double(s.a) + (double(s.b) + double(s.c)); }
+__device__ __forceinline__ double sum_value(Sum<double> s) { return s.a; }
 // lane 0: the sum over the warp
-template <typename R> __device__ __forceinline__ Pair<R> warp_join(Pair<R> v)
+__device__ __forceinline__ void warp_join(Sum<float> &s)
 {
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {
-        Pair<R> w;
-        w.h = __shfl_down_sync(0xffffffffu, v.h, o);
-        w.l = sizeof(R) == 4 ? __shfl_down_sync(0xffffffffu, v.l, o) : R(0);
-        v = pair_add(v, w);
+        const float a = __shfl_down_sync(0xffffffffu, s.a, o), b = __shfl_down_sync(0xffffffffu, s.b, o),
+                    c = __shfl_down_sync(0xffffffffu, s.c, o);
+        sum_add(s, a, b, c);
     }
-    return v;
+}
+__device__ __forceinline__ void warp_join(Sum<double> &s)
+{
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) s.a += __shfl_down_sync(0xffffffffu, s.a, o);
 }
 
 // (v0, v1) <- m (v0, v1), m row-major 2 x 2; complex64 with packed FMAs in cmac's order
@@ -634,7 +663,8 @@ __global__ void __launch_bounds__(kWindowThreads, 1) k_window(const __grid_const
                                                               typename C2<R>::type *__restrict__ psi)
 {
     using T2 = typename C2<R>::type;
-    __shared__ Pair<R> s_part[kWindowThreads / 32][kWindowRow];
+    __shared__ double s_part[kWindowThreads / 32][kWindowRow];
+    __shared__ Sum<R> s_sum[kWindowRow];
     __shared__ double s_rho[32], s_one[32], s_T[32], s_prob[kMaxKraus], s_M[2][32];
     __shared__ T2 s_m[2][16];
     __shared__ double s_op[2][3][kWindowOps], s_u[2];  // K, G, A of each channel
@@ -685,18 +715,15 @@ __global__ void __launch_bounds__(kWindowThreads, 1) k_window(const __grid_const
     if (p.na > 0) {
         // the CTAs' sums, in a fixed order: rows warp by warp, one column per lane
         const int width = p.na == 1 ? 6 : kWindowRow;
-        const Pair<R> *const in = reinterpret_cast<const Pair<R> *>(p.in);
-        Pair<R> part = {R(0), R(0)};
+        double part = 0;
         if (lane < width)
-            for (int r = warp; r < p.rows; r += kWindowThreads / 32)
-                part = pair_add(part, in[int64_t(r) * kWindowRow + lane]);
+            for (int r = warp; r < p.rows; r += kWindowThreads / 32) part += p.in[int64_t(r) * kWindowRow + lane];
         if (lane < kWindowRow) s_part[warp][lane] = part;
         __syncthreads();
         if (warp == 0) {
-            part = {R(0), R(0)};
+            double t = 0;
             if (lane < width)
-                for (int w = 0; w < kWindowThreads / 32; ++w) part = pair_add(part, s_part[w][lane]);
-            const double t = double(part.h) + double(part.l);
+                for (int w = 0; w < kWindowThreads / 32; ++w) t += s_part[w][lane];
             // upper triangle -> full matrix
             const int D = 1 << p.na;
             if (lane < width) {
@@ -854,16 +881,19 @@ __global__ void __launch_bounds__(kWindowThreads, 1) k_window(const __grid_const
             for (int b = 0; b < 2; ++b)
 #pragma unroll
                 for (int b2 = b; b2 < 2; ++b2, ++e) {
-                    T2 re, im;
-                    re.x = re.y = im.x = im.y = 0;
 #pragma unroll
-                    for (int a = 0; a < 8; ++a) {  // a: this window's qubits and the replaced one
-                        const T2 s = v[4 * (a >> 1) + 2 * b + (a & 1)], t = v[4 * (a >> 1) + 2 * b2 + (a & 1)];
-                        mac2(re, s, t);
-                        if (b != b2) mac2(im, swap_halves(s), t);
+                    for (int half = 0; half < 8; half += 4) {  // 8 products per compensated addition, as in k_rdm
+                        T2 re, im;
+                        re.x = re.y = im.x = im.y = 0;
+#pragma unroll
+                        for (int a = half; a < half + 4; ++a) {  // a: this window's qubits and the replaced one
+                            const T2 s = v[4 * (a >> 1) + 2 * b + (a & 1)], t = v[4 * (a >> 1) + 2 * b2 + (a & 1)];
+                            mac2(re, s, t);
+                            if (b != b2) mac2(im, swap_halves(s), t);
+                        }
+                        add(ar[e], cr[e], re.x + re.y);
+                        if (b != b2) add(ai[e], ci[e], im.x - im.y);
                     }
-                    add(ar[e], cr[e], re.x + re.y);
-                    if (b != b2) add(ai[e], ci[e], im.x - im.y);
                 }
         }
         f += stride;
@@ -871,23 +901,35 @@ __global__ void __launch_bounds__(kWindowThreads, 1) k_window(const __grid_const
     if constexpr (kStaged) cp_async_wait<0>();
     if (p.nb == 0) return;
     // every thread's sums to shared memory; lane by lane over the warps, then each sum's 32 lanes by shuffles (fixed
-    // order; five shuffle levels of all 20 sums in every warp took 3 us)
-    __syncthreads();
-    Pair<R> *const all = reinterpret_cast<Pair<R> *>(s_stage);  // [warp][sum][lane]
+    // order; five shuffle levels of all 20 sums in every warp took 3 us).  The barrier also tells whether a sum of the
+    // CTA is so large that joining it in FP32 could overflow: then all of them are scaled down first.
+    bool huge = false;
+    if constexpr (sizeof(R) == 4) {
+#pragma unroll
+        for (int e = 0; e < NE; ++e) huge = huge || fabsf(ar[e]) >= 0x1p100f || fabsf(ai[e]) >= 0x1p100f;
+    }
+    huge = __syncthreads_or(huge);
+    const R scale = huge ? R(0x1p-16) : R(1);
+    ThreadSum<R> *const all = reinterpret_cast<ThreadSum<R> *>(s_stage);  // [warp][sum][lane]
     const int width = p.nb == 1 ? 6 : kWindowRow;
 #pragma unroll
     for (int e = 0; e < NE; ++e)
         if (2 * e < width) {
-            all[(warp * kWindowRow + 2 * e) * 32 + lane] = pair_of(ar[e], cr[e]);
-            all[(warp * kWindowRow + 2 * e + 1) * 32 + lane] = pair_of(ai[e], ci[e]);
+            all[(warp * kWindowRow + 2 * e) * 32 + lane] = thread_sum(ar[e], cr[e], scale);
+            all[(warp * kWindowRow + 2 * e + 1) * 32 + lane] = thread_sum(ai[e], ci[e], scale);
         }
     __syncthreads();
     for (int j = warp; j < width; j += kWindowThreads / 32) {
-        Pair<R> t = all[j * 32 + lane];
-        for (int w = 1; w < kWindowThreads / 32; ++w) t = pair_add(t, all[(w * kWindowRow + j) * 32 + lane]);
-        t = warp_join(t);
-        if (lane == 0) reinterpret_cast<Pair<R> *>(p.out)[int64_t(blockIdx.x) * kWindowRow + j] = t;
+        Sum<R> t;
+        sum_start(t, all[j * 32 + lane]);
+        for (int w = 1; w < kWindowThreads / 32; ++w) sum_add(t, all[(w * kWindowRow + j) * 32 + lane]);
+        warp_join(t);
+        if (lane == 0) s_sum[j] = t;
     }
+    __syncthreads();
+    if (int(threadIdx.x) < width)
+        p.out[int64_t(blockIdx.x) * kWindowRow + threadIdx.x] =
+            sum_value(s_sum[threadIdx.x]) * (huge ? 0x1p16 : 1.0);
 }
 
 template <typename R> static int window_grid(int n)
@@ -927,7 +969,7 @@ template <typename R> static hq_status launch_window(const WindowParam &p, void 
 {
     // complex64: three stages of groups; then (and in complex128 only) the threads' sums
     const size_t smem = std::max(sizeof(R) == 4 ? size_t(3) * 16 * kWindowThreads * sizeof(float2) : size_t(0),
-                                 size_t(kWindowThreads) * kWindowRow * sizeof(Pair<R>));
+                                 size_t(kWindowThreads) * kWindowRow * sizeof(ThreadSum<R>));
     occupancy((const void *)k_window<R>, kWindowThreads, smem);  // (sets the kernel's shared-memory limit)
     k_window<R><<<window_grid<R>(n), kWindowThreads, smem, s>>>(p, (typename C2<R>::type *)state);
     return cuda_status("k_window", cudaGetLastError());
@@ -1077,7 +1119,7 @@ hq_status run_trajectory(void *state, int n, hq_dtype dt, const hq_noisy_op *ops
     for (const Dev &d : dev) hostbuf.push_back(u[d.ch]);
     // (n < 4: the per-channel kernels; a window kernel's threads hold four qubits)
     const bool windows = n >= 4;
-    const int width = windows ? kWindowRow * (dt == HQ_C64 ? 1 : 2) : 2 * rdm_entries<2>();  // doubles per row
+    const int width = windows ? kWindowRow : 2 * rdm_entries<2>();  // doubles per row
     const int grid = windows ? (dt == HQ_C64 ? window_grid<float>(n) : window_grid<double>(n))
                    : std::max(dt == HQ_C64 ? std::max(rdm_grid<float, 1>(n), rdm_grid<float, 2>(n))
                                            : std::max(rdm_grid<double, 1>(n), rdm_grid<double, 2>(n)), 1);
