@@ -12,6 +12,7 @@
 namespace hq {
 
 constexpr int kBlockTileMin = 9, kBlockTileMax = 13;  // tile bits a block pass takes
+constexpr int kBlocks3 = 8, kBlocks4 = 4;  // blocks of 3 and of 4 qubits per launch
 struct TileBlock {
     int k;
     int bit[4];        // flat bits, ascending; bit j of the matrix's index is bit[j]

@@ -326,8 +326,8 @@ void fuse_in_tile(int n, int K, uint64_t T, const hq_gate *gates, const std::vec
 hq_status launch_block_pass(void *state, int n, int L, uint64_t T, int K, std::vector<TileBlock> &blocks,
                             cudaStream_t s)
 {
-    if (K == 3) return launch_blocks<3, 8>(state, n, L, T, blocks, s);
-    return launch_blocks<4, 4>(state, n, L, T, blocks, s);
+    if (K == 3) return launch_blocks<3, kBlocks3>(state, n, L, T, blocks, s);
+    return launch_blocks<4, kBlocks4>(state, n, L, T, blocks, s);
 }
 
 }  // namespace hq

@@ -528,6 +528,8 @@ struct Item {
     bool swap;          // OP_D2: exchange the two qubits first
     uint16_t keep;      // OP_U2: bit 4 r + c set where the entry is not an exact zero
     uint64_t all, need; // flat bits; those that a register run mixes
+    double touched;     // share of the state that its own kernel reads and writes (below 1: k_ctrl)
+    bool perm;          // OP_BLK: one nonzero entry per row
     double m[8];        // matrix entries (U1: 2x2, D2 and PH: phases); OP_U2 and OP_DG read the gate's own
 };
 
@@ -553,11 +555,32 @@ int phase_kind(const double *e)
     return PHASE_ANY;
 }
 
-// max_block: the widest dense gate that a pass of blocks may take (2: none)
-void classify(int n, const hq_gate &g, int max_block, Item &it)
+// The share of the state that k_ctrl would read and write for this gate (1: not a controlled gate, or one that
+// k_ctrl does not take): half per control above the 32-byte sector.  Costs only, so without control_split's exact
+// tolerance.
+double touched_share(int n, const hq_gate &g, bool diagonal, int sector_bits)
+{
+    const int k = g.k, K = 1 << k;
+    int ctrl = K - 1;  // index bits that are 1 wherever the matrix differs from the identity
+    for (int r = 0; r < K && ctrl; ++r)
+        for (int c = diagonal ? r : 0; c < (diagonal ? r + 1 : K) && ctrl; ++c) {
+            const double *e = g.matrix + 2 * (r * K + c);
+            if (std::fabs(e[0] - (r == c ? 1.0 : 0.0)) > 1e-15 || std::fabs(e[1]) > 1e-15) ctrl &= r & c;
+        }
+    if (k - __builtin_popcount(unsigned(ctrl)) > kMaxCtrlTargets) return 1.0;
+    double share = 1.0;
+    for (int j = 0; j < k; ++j)
+        if (((ctrl >> (k - 1 - j)) & 1) && n - 1 - g.qubits[j] >= sector_bits) share *= 0.5;
+    return share;
+}
+
+// max_block: the widest dense gate that a pass of blocks may take (2: none); sector_bits: flat bits within 32 bytes
+void classify(int n, const hq_gate &g, int max_block, int sector_bits, Item &it)
 {
     const int k = g.k, K = 1 << k;
     const double *m = g.matrix;
+    it.touched = 1.0;
+    it.perm = false;
     it.wide = false;
     it.nb = uint8_t(k);
     it.all = it.need = 0;
@@ -570,6 +593,7 @@ void classify(int n, const hq_gate &g, int max_block, Item &it)
         it.all |= uint64_t(1) << it.bit[j];
     }
     if (is_diagonal(k, m)) {
+        it.touched = touched_share(n, g, true, sector_bits);
         bool phase = k <= 2;
         for (int r = 0; phase && r < K - 1; ++r)
             phase = m[2 * (r * K + r)] == 1.0 && m[2 * (r * K + r) + 1] == 0.0;
@@ -599,6 +623,14 @@ void classify(int n, const hq_gate &g, int max_block, Item &it)
         it.wide = k > max_block;
         it.pool = 0;
         it.need = it.all | kNever;
+        if (it.wide) return;
+        it.touched = touched_share(n, g, false, sector_bits);
+        it.perm = true;
+        for (int r = 0; r < K && it.perm; ++r) {
+            int nz = 0;
+            for (int c = 0; c < K && nz < 2; ++c) nz += m[2 * (r * K + c)] != 0.0 || m[2 * (r * K + c) + 1] != 0.0;
+            it.perm = nz == 1;
+        }
         return;
     }
     // k = 2: a controlled gate, an exchange with phases, or dense.  Entries within 4 FP64 epsilon of the largest
@@ -619,6 +651,7 @@ void classify(int n, const hq_gate &g, int max_block, Item &it)
         if (!ctrl) continue;
         const int tb = 3 ^ bit;
         it.kind = OP_U1;
+        if (n - 1 - g.qubits[j] >= sector_bits) it.touched = 0.5;
         it.pool = 16;  // 4, or 16 when the control is among the register bits
         it.target = int8_t(1 - j);
         it.need = uint64_t(1) << it.bit[1 - j];
@@ -915,13 +948,6 @@ bool compile_pass(PassParam<R> &p, int n, int L, uint64_t T, const std::vector<I
     return true;
 }
 
-// What the gate costs on its own kernel, in reads and writes of the state.
-double own_cost(const Item &i)
-{
-    if (i.kind == OP_PH) return i.nb == 1 ? 1.0 : 0.3;
-    return i.kind == OP_U1 && i.nb == 2 ? 0.55 : 1.0;
-}
-
 // Time of a gate in register runs and of a dense block in a block pass, ms at n = 28 (from whole circuits of 785 gates:
 // in runs 66.5 with CZ and 87 with fSim, in 139 three-qubit blocks 54.7, in 77 four-qubit blocks 59; QFT in runs); a
 // pass cannot take less than its read and write of the state.
@@ -937,6 +963,17 @@ double run_cost(const Item &i)
 }
 double block_cost(int K) { return K == 3 ? 0.39 : 0.77; }
 
+// complex64: the time of a gate on its own kernel, us.  Measured, n = 28 / 24 / 22 / 20: X 670 / 47 / 12 / 6.2, a
+// permutation of four qubits 703 / 49 / 13 / 6.3, a dense four-qubit gate 860 / 59 / 16 / 8; controlled gates by what k_ctrl
+// touches: CNOT 376 / 21 / 7 / 4.3, a controlled SWAP 375 / 22 / 8.6 / 4.6, Toffoli 180-224 / 11-14 / 6.2 / 4.2, one with
+// three controls 145 / 9 / 7.5 / 7.4 (the last ones by the host).
+double own_time(const Item &i, int n)
+{
+    const double full = i.kind == OP_BLK && i.nb == 4 && !i.perm ? 0.86 : 0.69;
+    const double ms = i.touched < 1.0 ? 0.04 + 0.63 * i.touched : full;  // n = 28
+    return std::max(4.2, 3.0 + std::ldexp(1e3 * ms, n - 28));
+}
+
 // complex128: the same for a gate in register runs and on its own kernel (ms at n = 28; FP64 multiply-adds at two per
 // clock and SM, 0.46 ms for one per amplitude; a read and write of the state 1.26 ms).  Measured at n = 22: a CNOT 43 us on
 // k_ctrl and 100 in runs (its 4 x 4 form tests every part), a dense two-qubit gate 154 and 157.
@@ -946,7 +983,7 @@ double own_cost_128(const Item &i)
     case OP_PH: return i.nb == 1 ? 1.85 : 0.5;
     case OP_U1: return i.nb == 2 ? 2.75 : 3.9;
     case OP_U2: return 9.8;
-    default: return 1.9;
+    default: return i.kind == OP_DG ? 0.1 + 1.8 * i.touched : 1.9;
     }
 }
 double run_cost_128(const Item &i)
@@ -965,6 +1002,7 @@ double run_cost_128(const Item &i)
     }
 }
 constexpr double kPassFloor = 0.75;
+constexpr double kPassLaunch = 7.0;  // us of a pass beside that (three gates of one qubit, n = 20: 9.8 us)
 // Below this size lists without 3- or 4-qubit gates stay on register runs (depth-12 CZ circuits, runs / blocks: n=25
 // 4.88 / 3.99 ms, n=23 1.28 / 1.20 ms; below, the plan of the blocks and their products cost the host more than that).
 constexpr int kBlockMinQubits = 23;
@@ -1074,17 +1112,37 @@ template <typename R, int RP> struct Segment {
                 std::memcpy(q.head, head, sizeof(int) * size_t(n));
             }
         }
-        double own = 0, own64 = 0, run64 = 0;
+        double own = 0, own64 = 0, run64 = 0, runs = 0, light = 0;
         bool dense = false;
         for (int g : list) {
             const Item &i = it[size_t(g)];
-            own += own_cost(i);
+            own += own_time(i, n);
+            // (a diagonal gate by its table: 0.185 of three qubits, 0.3 of six)
+            runs += i.kind == OP_DG ? 0.1 + 0.03 * i.nb : run_cost(i);
             dense = dense || i.kind == OP_U2;
-            if (sizeof(R) == 8) own64 += own_cost_128(i), run64 += run_cost_128(i);
+            if (sizeof(R) == 8) {
+                own64 += own_cost_128(i), run64 += run_cost_128(i);
+                light += i.kind == OP_PH && i.nb == 2 ? 0.3 : i.kind == OP_U1 && i.nb == 2 ? 0.55 : 1.0;
+            }
         }
-        if (list.size() == 1 || (n >= 20 && own <= 1.0)) kind = PASS_SINGLE;
+        if (list.size() == 1 || (sizeof(R) == 8 && n >= 20 && light <= 1.0)) kind = PASS_SINGLE;
+        // complex64, launches long enough to count: the pass only where it is the faster (a list of Toffoli gates, n =
+        // 28: 0.41 ms each in blocks, 0.18 to 0.22 on k_ctrl).  A pass with little work in it does not hide all of that
+        // under its copies (n = 28: three CZ 0.87, three one-qubit gates 1.01, two Toffoli gates 1.03 ms).
+        if (sizeof(R) == 4 && n >= 20) {
+            double cost = runs, launches = 1;
+            if (kind == PASS_BLOCKS) {
+                const int count = count_in_tile(n, K, gates, list), per = K == 3 ? kBlocks3 : kBlocks4;
+                launches = (count + per - 1) / per;
+                cost = block_cost(K) * count;
+            }
+            const double pass = std::max(cost, kPassFloor * launches + std::min(cost, 0.4));
+            if (own <= kPassLaunch * launches + std::ldexp(1e3 * pass, n - 28)) kind = PASS_SINGLE;
+        }
         // complex128: where the FP64 work of the gates is what counts, a pass saves nothing
-        if (sizeof(R) == 8 && (n >= 17 ? std::max(1.3, run64) >= 0.95 * own64 : list.size() <= 2 && dense))
+        // (n >= 22: a pass of three CZ 2.4 at n = 24 and 2.6 at n = 26, the three on k_ctrl 2.0 and 1.7)
+        if (sizeof(R) == 8 &&
+            (n >= 17 ? std::max(n >= 22 ? 2.4 : 1.3, run64) >= 0.95 * own64 : list.size() <= 2 && dense))
             kind = PASS_SINGLE;
         while (kind == PASS_RUNS && !compile_pass<R, RP>(p, n, L, T, it, gates, list)) {
             // too many runs: a shorter pass (the first half of the list is a valid order of its own)
@@ -1149,7 +1207,7 @@ hq_status run_list(void *state, int n, const hq_gate *gates, int G, int engine, 
         tile_shape<R>(n, L, c);
         // (4-qubit blocks: below 20 qubits their own kernel is faster, n=18 115 against 123 us for 19 blocks)
         const int max_block = sizeof(R) == 4 && L >= kBlockTileMin ? (n >= 20 ? 4 : 3) : 2;
-        for (int g = 0; g < cnt; ++g) classify(n, gs[g], max_block, it[size_t(g)]);
+        for (int g = 0; g < cnt; ++g) classify(n, gs[g], max_block, sizeof(R) == 4 ? 2 : 1, it[size_t(g)]);
         for (int g = 0; g < cnt;) {
             int e = g;
             while (e < cnt && !it[size_t(e)].wide) ++e;

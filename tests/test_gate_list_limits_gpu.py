@@ -48,3 +48,45 @@ def test_products_outside_the_float_range(hq, n, width, scale, dtype):
     top = float(want.abs().max())
     assert 0 < top < float("inf")
     assert float(torch.linalg.norm((got - want) / top)) <= tol * float(torch.linalg.norm(want / top))
+
+
+def controlled(U, controls):
+    m = np.eye(len(U) << controls, dtype=np.complex128)
+    m[-len(U):, -len(U):] = U
+    return m
+
+
+@pytest.mark.parametrize("form", ["ccx", "cccx", "cswap", "ccz", "perm4"])
+@pytest.mark.parametrize("n", [22, 25])
+def test_lists_of_controlled_gates(hq, n, form):
+    """Lists of gates that touch a part of the state on their own kernels: the
+    same state as one call at a time, and no list that runs at a fraction of
+    the single calls' speed."""
+    rng = np.random.default_rng(n)
+    m = {"ccx": controlled(C.PAULI["X"], 2), "cccx": controlled(C.PAULI["X"], 3), "cswap": controlled(C.swap(), 1),
+         "ccz": controlled(C.PAULI["Z"], 2), "perm4": np.eye(16, dtype=np.complex128)[rng.permutation(16)]}[form]
+    k = int(np.log2(len(m)))
+    gates = [C.Gate("a", tuple(int(q) for q in rng.choice(n, k, replace=False)), m) for _ in range(16)]
+    st = torch.randn(1 << n, dtype=torch.complex64, device="cuda")
+    one = st.clone()
+    singles = [[g] for g in gates]
+
+    def time(runs):
+        ms = []
+        for _ in range(7):
+            e = [torch.cuda.Event(enable_timing=True) for _ in range(2)]
+            torch.cuda._sleep(2_000_000)  # the host is ahead of the device
+            e[0].record()
+            for r in runs:
+                hq.hq_apply_blocks(st, r)
+            e[1].record()
+            torch.cuda.synchronize()
+            ms.append(e[0].elapsed_time(e[1]))
+        return min(ms)
+
+    hq.hq_apply_blocks(st, gates)
+    for g in gates:
+        hq.hq_apply_gate(one, g.qubits, g.matrix)
+    # exact products but for the sums of zeros and the order of disjoint gates: the same amplitudes
+    assert float(torch.linalg.norm(st - one)) <= 2e-6 * float(torch.linalg.norm(one))
+    assert time([gates]) <= 1.5 * time(singles)
