@@ -99,6 +99,36 @@ void make_geom(TileGeom &g, int n, int k, const int *qubits, int L, int64_t nsta
     g.state_stride = int64_t(1) << n;
 }
 
+// hypot(re, im) against a bound, the same answer as the call's, without it where |re| and |im| alone decide (gate
+// lists look at every matrix of every call: a six-qubit one has 4096 entries, 0.12 ms of hypot calls)
+static bool above(double re, double im, double bound)
+{
+    const double a = std::fabs(re), b = std::fabs(im);
+    if (a + b == a + b) {
+        if (a > 1.000001 * bound || b > 1.000001 * bound) return true;
+        if (a + b <= 0.999999 * bound) return false;
+    }
+    return std::hypot(re, im) > bound;
+}
+static bool within(double re, double im, double bound)
+{
+    const double a = std::fabs(re), b = std::fabs(im);
+    if (a + b == a + b) {
+        if (a > 1.000001 * bound || b > 1.000001 * bound) return false;
+        if (a + b <= 0.999999 * bound) return true;
+    }
+    return std::hypot(re, im) <= bound;
+}
+// the largest magnitude of the entries (NaN left out)
+static double largest(int k, const double *m)
+{
+    double mx = 0;
+    for (int e = 0; e < (1 << (2 * k)); ++e)
+        if (!(std::fabs(m[2 * e]) + std::fabs(m[2 * e + 1]) <= 0.999999 * mx))
+            mx = std::max(mx, std::hypot(m[2 * e], m[2 * e + 1]));
+    return mx;
+}
+
 // Monomial (permutation times diagonal): one nonzero per row and per column.
 // perm[r] = the column of row r's nonzero.  Entries below 4 epsilon (FP64) of
 // the largest magnitude count as zero: what they would add to a product is
@@ -107,14 +137,12 @@ void make_geom(TileGeom &g, int n, int k, const int *qubits, int L, int64_t nsta
 bool is_monomial(int k, const double *m, int *perm)
 {
     const int K = 1 << k;
-    double mx = 0;
-    for (int e = 0; e < K * K; ++e) mx = std::max(mx, std::hypot(m[2 * e], m[2 * e + 1]));
-    const double tiny = 4.0 * 2.220446049250313e-16 * mx;
+    const double tiny = 4.0 * 2.220446049250313e-16 * largest(k, m);
     int used = 0;
     for (int r = 0; r < K; ++r) {
         int col = -1;
         for (int c = 0; c < K; ++c)
-            if (std::hypot(m[2 * (r * K + c)], m[2 * (r * K + c) + 1]) > tiny) {
+            if (above(m[2 * (r * K + c)], m[2 * (r * K + c) + 1], tiny)) {
                 if (col >= 0) return false;
                 col = c;
             }
@@ -128,21 +156,17 @@ bool is_monomial(int k, const double *m, int *perm)
 int control_split(int k, const double *m, int *ctrl_mask, double *u)
 {
     const int K = 1 << k;
-    double mx = 0;
-    for (int e = 0; e < K * K; ++e) mx = std::max(mx, std::hypot(m[2 * e], m[2 * e + 1]));
-    const double tiny = 4.0 * 2.220446049250313e-16 * mx;
-    auto identity_entry = [&](int r, int c) {
-        return std::hypot(m[2 * (r * K + c)] - (r == c ? 1.0 : 0.0), m[2 * (r * K + c) + 1]) <= tiny;
-    };
+    const double tiny = 4.0 * 2.220446049250313e-16 * largest(k, m);
+    // a control: its bit is 1 in the row and the column of every entry that differs from the identity's
+    int bits = K - 1;
+    for (int r = 0; r < K && bits; ++r)
+        for (int c = 0; c < K && bits; ++c)
+            if ((r & c & bits) != bits &&
+                !within(m[2 * (r * K + c)] - (r == c ? 1.0 : 0.0), m[2 * (r * K + c) + 1], tiny))
+                bits &= r & c;
     int cm = 0;
-    for (int j = 0; j < k; ++j) {
-        const int bit = 1 << (k - 1 - j);
-        bool ok = true;
-        for (int r = 0; r < K && ok; ++r)
-            for (int c = 0; c < K && ok; ++c)
-                if (!(r & bit) || !(c & bit)) ok = identity_entry(r, c);
-        if (ok) cm |= 1 << j;
-    }
+    for (int j = 0; j < k; ++j)
+        if (bits & (1 << (k - 1 - j))) cm |= 1 << j;
     *ctrl_mask = cm;
     if (u) {
         int tq[HQ_MAX_K], kt = 0, all = 0;
