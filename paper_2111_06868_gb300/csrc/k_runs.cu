@@ -1112,7 +1112,7 @@ template <typename R, int RP> struct Segment {
                 std::memcpy(q.head, head, sizeof(int) * size_t(n));
             }
         }
-        double own = 0, own64 = 0, run64 = 0, runs = 0, light = 0;
+        double own = 0, own64 = 0, run64 = 0, runs = 0, light = 0, few_own = 0, few_run = 0;
         bool dense = false;
         for (int g : list) {
             const Item &i = it[size_t(g)];
@@ -1121,6 +1121,9 @@ template <typename R, int RP> struct Segment {
             runs += i.kind == OP_DG ? 0.1 + 0.03 * i.nb : run_cost(i);
             dense = dense || i.kind == OP_U2;
             if (sizeof(R) == 8) {
+                const bool full = i.kind == OP_U2 && i.keep == 0xffff;
+                few_own += full ? 6.2 : 4.1;
+                few_run += i.kind == OP_U2 ? 4.9 : i.kind == OP_U1 && i.nb == 2 ? 3.3 : 1.0;
                 own64 += own_cost_128(i), run64 += run_cost_128(i);
                 light += i.kind == OP_PH && i.nb == 2 ? 0.3 : i.kind == OP_U1 && i.nb == 2 ? 0.55 : 1.0;
             }
@@ -1144,6 +1147,9 @@ template <typename R, int RP> struct Segment {
         if (sizeof(R) == 8 &&
             (n >= 17 ? std::max(n >= 22 ? 2.4 : 1.3, run64) >= 0.95 * own64 : list.size() <= 2 && dense))
             kind = PASS_SINGLE;
+        // complex128 on up to 9 qubits: one CTA, a gate takes its FP64 latency (16 permutations of two qubits, n = 6 / 9: 83
+        // / 80 us in runs, 66 in launches; two CNOT, n = 8: 10.6 and 8.2)
+        if (sizeof(R) == 8 && n <= 9 && few_own <= 4.0 + few_run) kind = PASS_SINGLE;
         while (kind == PASS_RUNS && !compile_pass<R, RP>(p, n, L, T, it, gates, list)) {
             // too many runs: a shorter pass (the first half of the list is a valid order of its own)
             list.resize(list.size() / 2);
