@@ -656,14 +656,17 @@ __device__ __forceinline__ void mac2(double2 &acc, double2 a, double2 b)
 constexpr int kWindowOps = 64;  // doubles of K (and of G) that are staged in shared memory
 
 // one CTA per SM: few partial sums to read back (152 rows instead of 304: the pick's FP64 additions halve twice over)
-constexpr int kWindowThreads = 512;
+// (512 threads; complex128 on states with few groups of 16 amplitudes, bound by the FP64 latency of an SM quarter's
+// warps: 128, so that the groups reach four times as many SMs: a channel alone, n = 14 / 18 / 19, 102 / 106 / 118 us with
+// 512 threads, 72 / 77 / 94 with 128; k_rdm, k_kraus_pick and k_apply_sel took 87 / 92 / 119)
+constexpr int kWindowMany = 512, kWindowFew = 128;
 
-template <typename R>
-__global__ void __launch_bounds__(kWindowThreads, 1) k_window(const __grid_constant__ WindowParam p,
+template <typename R, int TH>
+__global__ void __launch_bounds__(TH, 1) k_window(const __grid_constant__ WindowParam p,
                                                               typename C2<R>::type *__restrict__ psi)
 {
     using T2 = typename C2<R>::type;
-    __shared__ double s_part[kWindowThreads / 32][kWindowRow];
+    __shared__ double s_part[TH / 32][kWindowRow];
     __shared__ Sum<R> s_sum[kWindowRow];
     __shared__ double s_rho[32], s_one[32], s_T[32], s_prob[kMaxKraus], s_M[2][32];
     __shared__ T2 s_m[2][16];
@@ -685,7 +688,7 @@ __global__ void __launch_bounds__(kWindowThreads, 1) k_window(const __grid_const
     // Three stages: a stage is filled again only after the arithmetic on what was read from it.
     constexpr bool kStaged = sizeof(R) == 4;
     extern __shared__ __align__(16) unsigned char s_stage[];
-    T2 *const slot = reinterpret_cast<T2 *>(s_stage) + threadIdx.x;  // [stage][16][kWindowThreads]
+    T2 *const slot = reinterpret_cast<T2 *>(s_stage) + threadIdx.x;  // [stage][16][TH]
     T2 v[16];
     int64_t f = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
     int stage = 0;
@@ -693,7 +696,7 @@ __global__ void __launch_bounds__(kWindowThreads, 1) k_window(const __grid_const
         if (g < groups) {
             const T2 *const from = psi + spread(g);
 #pragma unroll
-            for (int i = 0; i < 16; ++i) cp_async8(slot + (16 * to + i) * kWindowThreads, from + p.off[i]);
+            for (int i = 0; i < 16; ++i) cp_async8(slot + (16 * to + i) * TH, from + p.off[i]);
         }
         cp_async_commit();
     };
@@ -717,13 +720,13 @@ __global__ void __launch_bounds__(kWindowThreads, 1) k_window(const __grid_const
         const int width = p.na == 1 ? 6 : kWindowRow;
         double part = 0;
         if (lane < width)
-            for (int r = warp; r < p.rows; r += kWindowThreads / 32) part += p.in[int64_t(r) * kWindowRow + lane];
+            for (int r = warp; r < p.rows; r += TH / 32) part += p.in[int64_t(r) * kWindowRow + lane];
         if (lane < kWindowRow) s_part[warp][lane] = part;
         __syncthreads();
         if (warp == 0) {
             double t = 0;
             if (lane < width)
-                for (int w = 0; w < kWindowThreads / 32; ++w) t += s_part[w][lane];
+                for (int w = 0; w < TH / 32; ++w) t += s_part[w][lane];
             // upper triangle -> full matrix
             const int D = 1 << p.na;
             if (lane < width) {
@@ -821,7 +824,7 @@ __global__ void __launch_bounds__(kWindowThreads, 1) k_window(const __grid_const
         if constexpr (kStaged) {
             cp_async_wait<1>();
 #pragma unroll
-            for (int i = 0; i < 16; ++i) v[i] = slot[(16 * stage + i) * kWindowThreads];
+            for (int i = 0; i < 16; ++i) v[i] = slot[(16 * stage + i) * TH];
             fetch(f + 2 * stride, stage == 0 ? 2 : stage - 1);
             stage = stage == 2 ? 0 : stage + 1;
         } else {
@@ -919,10 +922,10 @@ __global__ void __launch_bounds__(kWindowThreads, 1) k_window(const __grid_const
             all[(warp * kWindowRow + 2 * e + 1) * 32 + lane] = thread_sum(ai[e], ci[e], scale);
         }
     __syncthreads();
-    for (int j = warp; j < width; j += kWindowThreads / 32) {
+    for (int j = warp; j < width; j += TH / 32) {
         Sum<R> t;
         sum_start(t, all[j * 32 + lane]);
-        for (int w = 1; w < kWindowThreads / 32; ++w) sum_add(t, all[(w * kWindowRow + j) * 32 + lane]);
+        for (int w = 1; w < TH / 32; ++w) sum_add(t, all[(w * kWindowRow + j) * 32 + lane]);
         warp_join(t);
         if (lane == 0) s_sum[j] = t;
     }
@@ -932,10 +935,15 @@ __global__ void __launch_bounds__(kWindowThreads, 1) k_window(const __grid_const
             sum_value(s_sum[threadIdx.x]) * (huge ? 0x1p16 : 1.0);
 }
 
-template <typename R> static int window_grid(int n)
+static int window_threads(int n, hq_dtype dt)
+{
+    return dt == HQ_C128 && (int64_t(1) << (n - 4)) <= int64_t(sm_count()) * 2 * kWindowFew ? kWindowFew : kWindowMany;
+}
+static int window_grid(int n, hq_dtype dt)
 {
     const int64_t groups = int64_t(1) << (n - 4);
-    return int(std::min<int64_t>(sm_count(), (groups + kWindowThreads - 1) / kWindowThreads));
+    const int threads = window_threads(n, dt);
+    return int(std::min<int64_t>(sm_count(), (groups + threads - 1) / threads));
 }
 
 // the bits a window kernel works on: this window's qubits a, the next one's b, others in the place of missing ones
@@ -965,14 +973,21 @@ static void window_bits(WindowParam &p, int n, int na, const int *qa, int nb, co
     p.nb = nb;
 }
 
-template <typename R> static hq_status launch_window(const WindowParam &p, void *state, int n, cudaStream_t s)
+template <typename R, int TH> static hq_status launch_window_as(const WindowParam &p, void *state, int grid, cudaStream_t s)
 {
     // complex64: three stages of groups; then (and in complex128 only) the threads' sums
-    const size_t smem = std::max(sizeof(R) == 4 ? size_t(3) * 16 * kWindowThreads * sizeof(float2) : size_t(0),
-                                 size_t(kWindowThreads) * kWindowRow * sizeof(ThreadSum<R>));
-    occupancy((const void *)k_window<R>, kWindowThreads, smem);  // (sets the kernel's shared-memory limit)
-    k_window<R><<<window_grid<R>(n), kWindowThreads, smem, s>>>(p, (typename C2<R>::type *)state);
+    const size_t smem = std::max(sizeof(R) == 4 ? size_t(3) * 16 * TH * sizeof(float2) : size_t(0),
+                                 size_t(TH) * kWindowRow * sizeof(ThreadSum<R>));
+    occupancy((const void *)k_window<R, TH>, TH, smem);  // (sets the kernel's shared-memory limit)
+    k_window<R, TH><<<grid, TH, smem, s>>>(p, (typename C2<R>::type *)state);
     return cuda_status("k_window", cudaGetLastError());
+}
+static hq_status launch_window(const WindowParam &p, void *state, int n, hq_dtype dt, cudaStream_t s)
+{
+    const int grid = window_grid(n, dt);
+    if (dt == HQ_C64) return launch_window_as<float, kWindowMany>(p, state, grid, s);
+    if (window_threads(n, dt) == kWindowFew) return launch_window_as<double, kWindowFew>(p, state, grid, s);
+    return launch_window_as<double, kWindowMany>(p, state, grid, s);
 }
 
 // K^dag K as a row-major D x D complex matrix
@@ -1120,7 +1135,7 @@ hq_status run_trajectory(void *state, int n, hq_dtype dt, const hq_noisy_op *ops
     // (n < 4: the per-channel kernels; a window kernel's threads hold four qubits)
     const bool windows = n >= 4;
     const int width = windows ? kWindowRow : 2 * rdm_entries<2>();  // doubles per row
-    const int grid = windows ? (dt == HQ_C64 ? window_grid<float>(n) : window_grid<double>(n))
+    const int grid = windows ? window_grid(n, dt)
                    : std::max(dt == HQ_C64 ? std::max(rdm_grid<float, 1>(n), rdm_grid<float, 2>(n))
                                            : std::max(rdm_grid<double, 1>(n), rdm_grid<double, 2>(n)), 1);
     // two sets of partial sums: a window kernel writes the next one's while other CTAs still read its own
@@ -1211,7 +1226,7 @@ hq_status run_trajectory(void *state, int n, hq_dtype dt, const hq_noisy_op *ops
                 std::memset(&w, 0, sizeof(w));
                 window_bits(w, n, 0, nullptr, na, qa);
                 w.out = partials + size_t(side) * grid * width;
-                st = dt == HQ_C64 ? launch_window<float>(w, state, n, s) : launch_window<double>(w, state, n, s);
+                st = launch_window(w, state, n, dt, s);
                 if (st != HQ_OK) break;
             }
             std::memset(&w, 0, sizeof(w));
@@ -1232,7 +1247,7 @@ hq_status run_trajectory(void *state, int n, hq_dtype dt, const hq_noisy_op *ops
             w.rows = grid;
             side ^= 1;
             w.out = partials + size_t(side) * grid * width;
-            st = dt == HQ_C64 ? launch_window<float>(w, state, n, s) : launch_window<double>(w, state, n, s);
+            st = launch_window(w, state, n, dt, s);
             fed = nb > 0;
             done = size_t(last) + 1;
             ++di;
