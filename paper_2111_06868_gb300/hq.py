@@ -229,7 +229,7 @@ def _gates_array(gates: Iterable, keep: list):
         k = len(qs)
         try:
             _PACK_GATE[k].pack_into(arr, at, k, *qs, p)
-        except (struct.error, IndexError):  # qubits that are not integers but convert to them; too many
+        except (struct.error, TypeError, IndexError):  # qubits that are not integers but convert to them; too many
             arr[i] = _gate_struct(qs, m, keep)
         at += _GATE_BYTES
     return arr, len(gl)
@@ -488,7 +488,7 @@ def hq_run_trajectory(state, ops, u, engine: str | int = "auto", tc_min_k: int =
         k = len(qubits)
         try:
             _PACK_NOISY[k].pack_into(arr, i * _NOISY_BYTES, k, *qubits, nk, p)
-        except (struct.error, IndexError):
+        except (struct.error, TypeError, IndexError):
             h = arr[i]
             h.k = k
             for j, q in enumerate(qubits):
