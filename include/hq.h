@@ -54,7 +54,7 @@ typedef int hq_status;
 #define HQ_ERR_K_TOO_LARGE (-4)  /* k < 1 or k > HQ_MAX_K, or k > n */
 #define HQ_ERR_N_TOO_LARGE (-5)  /* n < 1 or n > HQ_MAX_N */
 #define HQ_ERR_DTYPE (-6)        /* unknown hq_dtype, or dtype not supported by the engine */
-#define HQ_ERR_ALLOC (-7)        /* device scratch allocation failed */
+#define HQ_ERR_ALLOC (-7)        /* device scratch (or host memory) allocation failed */
 #define HQ_ERR_CUDA (-8)         /* a CUDA runtime call failed */
 #define HQ_ERR_TIMEOUT (-9)      /* a bounded device-side wait ran out */
 #define HQ_ERR_TOKEN (-10)       /* initial-state token not in {0,1,+,-} */
@@ -447,8 +447,9 @@ hq_status hq_apply_gate(void *state, int n, hq_dtype dt, const int *qubits, int 
  * On HQ_ERR_ALLOC the state is left as follows: the tensor-core engines and
  * HQ_ENGINE_TC_PASS take their one scratch buffer before enqueueing any
  * kernel, so the state is untouched; HQ_ENGINE_AUTO / HQ_ENGINE_CUDA_CORE
- * allocate per wide (k = 5, 6) block, so the blocks before the one whose
- * allocation failed have been applied and none after it.
+ * allocate per wide (k = 5, 6) block, and host memory for the plan at the start
+ * of a run of narrower gates (and every 4096 gates), so the gates before the
+ * block or run whose allocation failed have been applied and none after it.
  */
 hq_status hq_apply_blocks(void *state, int n, hq_dtype dt, const hq_gate *gates, int G, const hq_config *cfg,
                           void *stream);

@@ -4,6 +4,7 @@
 #include <cstdio>
 #include <cstring>
 #include <mutex>
+#include <new>
 #include <string>
 #include <vector>
 
@@ -13,12 +14,25 @@ namespace hq {
 
 static thread_local std::string t_last_error;
 
+// (the text is lost when there is no host memory for it: no exception leaves the library)
 void set_last_error(const char *what, cudaError_t e)
 {
-    t_last_error = std::string(what) + ": " + cudaGetErrorName(e) + " (" + cudaGetErrorString(e) + ")";
+    try {
+        t_last_error = std::string(what) + ": " + cudaGetErrorName(e) + " (" + cudaGetErrorString(e) + ")";
+    } catch (const std::bad_alloc &) {
+        t_last_error.clear();
+    }
 }
 
 void set_last_error_text(const std::string &text) { t_last_error = text; }
+void set_last_error_text(const char *text) noexcept
+{
+    try {
+        t_last_error = text;
+    } catch (const std::bad_alloc &) {
+        t_last_error.clear();
+    }
+}
 
 hq_status cuda_status(const char *what, cudaError_t e)
 {

@@ -19,14 +19,23 @@ struct TileBlock {
     double m[2 * 256]; // 2^k x 2^k complex, row-major
 };
 
-// The listed gates (a valid order, every qubit in the tile T, none wider than
-// K = 3 or 4) fused into blocks of exactly K qubits.
-void fuse_in_tile(int n, int K, uint64_t T, const hq_gate *gates, const std::vector<int> &list,
-                  std::vector<TileBlock> &blocks);
-// The number of blocks that makes.
-int count_in_tile(int n, int K, const hq_gate *gates, const std::vector<int> &list);
-// The blocks in order on a complex64 state, tiles of the L bits T.
-hq_status launch_block_pass(void *state, int n, int L, uint64_t T, int K, std::vector<TileBlock> &blocks,
-                            cudaStream_t s);
+// What planning and fusing a pass writes: reserved for every gate of a list's segment before its first launch, so that
+// no pass allocates.
+struct BlockScratch {
+    std::vector<uint64_t> set;
+    std::vector<int> member;
+    void reserve(size_t gates)
+    {
+        set.reserve(gates);
+        member.reserve(gates);
+    }
+};
+
+// The number of blocks of at most K = 3 or 4 qubits that the listed gates (a valid order, none wider than K) make.
+int count_in_tile(int n, int K, const hq_gate *gates, const std::vector<int> &list, BlockScratch &sc);
+// The listed gates, every qubit in the tile T of L bits, fused into blocks of K qubits and applied in order to a
+// complex64 state.
+hq_status launch_block_pass(void *state, int n, int L, uint64_t T, int K, const hq_gate *gates,
+                            const std::vector<int> &list, BlockScratch &sc, cudaStream_t s);
 
 }  // namespace hq

@@ -16,6 +16,7 @@ namespace hq {
 // ----------------------------------------------------------------------------
 void set_last_error(const char *what, cudaError_t e);
 void set_last_error_text(const std::string &text);
+void set_last_error_text(const char *text) noexcept;
 hq_status cuda_status(const char *what, cudaError_t e);  // HQ_OK or HQ_ERR_CUDA
 #define HQ_CUDA(call)                                              \
     do {                                                           \

@@ -34,6 +34,7 @@
 #include <cstring>
 #include <map>
 #include <mutex>
+#include <new>
 #include <vector>
 
 #include "hq_cp_async.cuh"
@@ -231,17 +232,27 @@ int occupancy(const void *fn, int threads, size_t smem)
     int dev = 0;
     cudaGetDevice(&dev);
     std::lock_guard<std::mutex> lk(g_occ_mu);
-    size_t &lim = g_smem_limit[std::make_pair(dev, fn)];
-    if (smem > 48 * 1024 && smem > lim) {
-        cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
-        lim = smem;
+    // (out of host memory: looked up again next time, so that no launch of a list fails for it)
+    if (smem > 48 * 1024) {
+        const auto key = std::make_pair(dev, fn);
+        auto it = g_smem_limit.find(key);
+        if (it == g_smem_limit.end() || smem > it->second) {
+            cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
+            try {
+                g_smem_limit[key] = smem;
+            } catch (const std::bad_alloc &) {
+            }
+        }
     }
-    auto key = std::make_pair(dev * 1024 + int(smem >> 10), fn);
+    const auto key = std::make_pair(dev * 1024 + int(smem >> 10), fn);
     auto it = g_occ.find(key);
     if (it != g_occ.end()) return it->second;
     int nb = 0;
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, fn, threads, smem) != cudaSuccess || nb < 1) nb = 1;
-    g_occ[key] = nb;
+    try {
+        g_occ[key] = nb;
+    } catch (const std::bad_alloc &) {
+    }
     return nb;
 }
 

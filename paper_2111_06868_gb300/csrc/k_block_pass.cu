@@ -19,7 +19,6 @@
 // n = 28, 785-gate fSim circuit: 87 ms in register runs, 54.7 in 139 three-qubit blocks (25 passes).  Lists of
 // 4-qubit blocks, n = 28: 64.1 ms one launch per block (k_gather_pair), 59.3 in passes; 3-qubit blocks n = 24: 3.72 -> 2.00
 // ms, n = 12: 213 -> 67 us.
-#include <algorithm>
 #include <cmath>
 #include <cstring>
 #include <vector>
@@ -219,13 +218,70 @@ bool float_range(const TileBlock &blk, int K)
     return true;
 }
 
+// sc.set: the qubits of each block; sc.member: the block of each listed gate
+void group_in_tile(int n, int K, const hq_gate *gates, const std::vector<int> &list, BlockScratch &sc)
+{
+    sc.set.clear();
+    sc.member.clear();
+    for (int g : list) {
+        uint64_t q = 0;
+        for (int j = 0; j < gates[g].k; ++j) q |= uint64_t(1) << (n - 1 - gates[g].qubits[j]);
+        // the latest block that shares a qubit when the union fits, else the first later one that fits, else a new one
+        int i = int(sc.set.size()) - 1, to = -1;
+        while (i >= 0 && !(sc.set[size_t(i)] & q)) --i;
+        if (i >= 0 && __builtin_popcountll(sc.set[size_t(i)] | q) <= K) to = i;
+        for (int j = i + 1; to < 0 && j < int(sc.set.size()); ++j)
+            if (__builtin_popcountll(sc.set[size_t(j)] | q) <= K) to = j;
+        if (to < 0) {
+            sc.set.push_back(0);
+            to = int(sc.set.size()) - 1;
+        }
+        sc.set[size_t(to)] |= q;
+        sc.member.push_back(to);
+    }
+}
+
+// The listed gates (a valid order, every qubit in the tile T, none wider than K) fused into blocks of exactly K
+// qubits; emit(block) for each in order, until one returns an error.
+template <typename Emit>
+hq_status fuse_in_tile(int n, int K, uint64_t T, const hq_gate *gates, const std::vector<int> &list, BlockScratch &sc,
+                       Emit emit)
+{
+    group_in_tile(n, K, gates, list, sc);
+    TileBlock blk;
+    hq_status st = HQ_OK;
+    for (size_t b = 0; b < sc.set.size() && st == HQ_OK; ++b) {
+        // a block of fewer qubits is widened by the tile's highest other bits (identity there)
+        uint64_t set = sc.set[b];
+        for (int x = 63; x >= 0 && __builtin_popcountll(set) < K; --x)
+            if (((T >> x) & 1) && !((set >> x) & 1)) set |= uint64_t(1) << x;
+        identity_block(blk, K, set);
+        for (size_t i = 0; i < list.size(); ++i)
+            if (sc.member[i] == int(b)) multiply_in(blk, K, n, gates[list[i]]);
+        if (float_range(blk, K)) {
+            st = emit(blk);
+            continue;
+        }
+        // the product leaves FP32's range where its gates need not: one block per gate
+        for (size_t i = 0; i < list.size() && st == HQ_OK; ++i)
+            if (sc.member[i] == int(b)) {
+                identity_block(blk, K, set);
+                multiply_in(blk, K, n, gates[list[i]]);
+                st = emit(blk);
+            }
+    }
+    return st;
+}
+
 template <int K, int NB>
-hq_status launch_blocks(void *state, int n, int L, uint64_t T, std::vector<TileBlock> &blocks, cudaStream_t s)
+hq_status launch_blocks(void *state, int n, int L, uint64_t T, const hq_gate *gates, const std::vector<int> &list,
+                        BlockScratch &sc, cudaStream_t s)
 {
     constexpr int D = 1 << K;
     BlockPassParam<K, NB> p;
     p.n = n;
     p.L = L;
+    p.nb = 0;
     int pos[HQ_MAX_N], m = 0, c = 0;
     while (c < n && ((T >> c) & 1)) ++c;
     p.c = c;
@@ -234,100 +290,48 @@ hq_status launch_blocks(void *state, int n, int L, uint64_t T, std::vector<TileB
             if (m >= c) p.hi[m - c] = uint8_t(b);
             pos[b] = m++;
         }
-    for (size_t first = 0; first < blocks.size(); first += NB) {
-        p.nb = int(std::min<size_t>(NB, blocks.size() - first));
-        for (int b = 0; b < p.nb; ++b) {
-            const TileBlock &blk = blocks[first + size_t(b)];
-            for (int j = 0; j < K; ++j) p.asc[b][j] = pos[blk.bit[j]];  // (ascending as the flat bits are)
-            for (int r = 0; r < D; ++r) {
-                int i = 0;
-                for (int j = 0; j < K; ++j)
-                    if ((r >> j) & 1) i |= 1 << p.asc[b][j];
-                p.off[b][r] = bswz(i) * int(sizeof(float2));
-                for (int x = 0; x < D; ++x) {
-                    const double *e = blk.m + 2 * (r * D + x);
-                    const float re[2] = {float(e[0]), float(e[0])}, im[2] = {float(e[1]), float(e[1])};
-                    std::memcpy(&p.a[b][r][x].x, re, 8);
-                    std::memcpy(&p.a[b][r][x].y, im, 8);
-                }
-            }
-        }
+    auto launch = [&]() -> hq_status {
         const size_t smem = sizeof(float2) << L;
         const void *fn = (const void *)k_block_pass<K, NB>;
         const int grid = grid_for(fn, kBpThreads, smem, int64_t(1) << (n - L));
         k_block_pass<K, NB><<<grid, kBpThreads, smem, s>>>(p, (float2 *)state);
-        hq_status st = cuda_status("k_block_pass", cudaGetLastError());
-        if (st != HQ_OK) return st;
-    }
-    return HQ_OK;
+        p.nb = 0;
+        return cuda_status("k_block_pass", cudaGetLastError());
+    };
+    // NB blocks at a time: the first launch runs while the host multiplies the next ones
+    hq_status st = fuse_in_tile(n, K, T, gates, list, sc, [&](const TileBlock &blk) -> hq_status {
+        const int b = p.nb++;
+        for (int j = 0; j < K; ++j) p.asc[b][j] = pos[blk.bit[j]];  // (ascending as the flat bits are)
+        for (int r = 0; r < D; ++r) {
+            int i = 0;
+            for (int j = 0; j < K; ++j)
+                if ((r >> j) & 1) i |= 1 << p.asc[b][j];
+            p.off[b][r] = bswz(i) * int(sizeof(float2));
+            for (int x = 0; x < D; ++x) {
+                const double *e = blk.m + 2 * (r * D + x);
+                const float re[2] = {float(e[0]), float(e[0])}, im[2] = {float(e[1]), float(e[1])};
+                std::memcpy(&p.a[b][r][x].x, re, 8);
+                std::memcpy(&p.a[b][r][x].y, im, 8);
+            }
+        }
+        return p.nb == NB ? launch() : HQ_OK;
+    });
+    return st == HQ_OK && p.nb > 0 ? launch() : st;
 }
 
 }  // namespace
 
-// set: the qubits of each block; member: the block of each listed gate
-static void group_in_tile(int n, int K, const hq_gate *gates, const std::vector<int> &list,
-                          std::vector<uint64_t> &set, std::vector<int> &member)
+int count_in_tile(int n, int K, const hq_gate *gates, const std::vector<int> &list, BlockScratch &sc)
 {
-    set.clear();
-    member.clear();
-    for (int g : list) {
-        uint64_t q = 0;
-        for (int j = 0; j < gates[g].k; ++j) q |= uint64_t(1) << (n - 1 - gates[g].qubits[j]);
-        // the latest block that shares a qubit when the union fits, else the first later one that fits, else a new one
-        int i = int(set.size()) - 1, to = -1;
-        while (i >= 0 && !(set[size_t(i)] & q)) --i;
-        if (i >= 0 && __builtin_popcountll(set[size_t(i)] | q) <= K) to = i;
-        for (int j = i + 1; to < 0 && j < int(set.size()); ++j)
-            if (__builtin_popcountll(set[size_t(j)] | q) <= K) to = j;
-        if (to < 0) {
-            set.push_back(0);
-            to = int(set.size()) - 1;
-        }
-        set[size_t(to)] |= q;
-        member.push_back(to);
-    }
+    group_in_tile(n, K, gates, list, sc);
+    return int(sc.set.size());
 }
 
-int count_in_tile(int n, int K, const hq_gate *gates, const std::vector<int> &list)
+hq_status launch_block_pass(void *state, int n, int L, uint64_t T, int K, const hq_gate *gates,
+                            const std::vector<int> &list, BlockScratch &sc, cudaStream_t s)
 {
-    std::vector<uint64_t> set;
-    std::vector<int> member;
-    group_in_tile(n, K, gates, list, set, member);
-    return int(set.size());
-}
-
-void fuse_in_tile(int n, int K, uint64_t T, const hq_gate *gates, const std::vector<int> &list,
-                  std::vector<TileBlock> &blocks)
-{
-    blocks.clear();
-    std::vector<uint64_t> set;
-    std::vector<int> member;
-    group_in_tile(n, K, gates, list, set, member);
-    for (size_t b = 0; b < set.size(); ++b) {
-        // a block of fewer qubits is widened by the tile's highest other bits (identity there)
-        for (int x = 63; x >= 0 && __builtin_popcountll(set[b]) < K; --x)
-            if (((T >> x) & 1) && !((set[b] >> x) & 1)) set[b] |= uint64_t(1) << x;
-        blocks.emplace_back();
-        identity_block(blocks.back(), K, set[b]);
-        for (size_t i = 0; i < list.size(); ++i)
-            if (member[i] == int(b)) multiply_in(blocks.back(), K, n, gates[list[i]]);
-        if (float_range(blocks.back(), K)) continue;
-        // the product leaves FP32's range where its gates need not: one block per gate
-        blocks.pop_back();
-        for (size_t i = 0; i < list.size(); ++i)
-            if (member[i] == int(b)) {
-                blocks.emplace_back();
-                identity_block(blocks.back(), K, set[b]);
-                multiply_in(blocks.back(), K, n, gates[list[i]]);
-            }
-    }
-}
-
-hq_status launch_block_pass(void *state, int n, int L, uint64_t T, int K, std::vector<TileBlock> &blocks,
-                            cudaStream_t s)
-{
-    if (K == 3) return launch_blocks<3, kBlocks3>(state, n, L, T, blocks, s);
-    return launch_blocks<4, kBlocks4>(state, n, L, T, blocks, s);
+    if (K == 3) return launch_blocks<3, kBlocks3>(state, n, L, T, gates, list, sc, s);
+    return launch_blocks<4, kBlocks4>(state, n, L, T, gates, list, sc, s);
 }
 
 }  // namespace hq

@@ -770,14 +770,27 @@ void put_entry(PassParam<R> &p, int at, const double *e)
     p.pool[at].y = R(e[1]);
 }
 
-// Groups the pass's gates (in a valid order) into register runs and writes the
+// What planning a pass writes; as BlockScratch, reserved for a whole segment before its first launch: a list that runs
+// out of host memory leaves the state after one of its gates, not amid a pass's reordered ones.
+struct PlanScratch {
+    std::vector<int> todo, rest, taken, blist;
+    BlockScratch block;
+    void reserve(size_t gates)
+    {
+        for (std::vector<int> *v : {&todo, &rest, &taken, &blist}) v->reserve(gates);
+        block.reserve(gates);
+    }
+};
+
+// Groups the pass's gates (sc.todo, in a valid order) into register runs and writes the
 // kernel's parameters.  T: the tile's flat bits (L of them, the lowest c
 // contiguous).  False when the runs do not fit (the caller then shortens the
 // list).
 template <typename R, int RP>
 bool compile_pass(PassParam<R> &p, int n, int L, uint64_t T, const std::vector<Item> &it, const hq_gate *gates,
-                  std::vector<int> list)
+                  PlanScratch &sc)
 {
+    std::vector<int> &list = sc.todo, &rest = sc.rest, &taken = sc.taken;
     constexpr int NB = Traits<R>::NB, NA = 1 << RP;
     p.n = n;
     p.L = L;
@@ -794,7 +807,6 @@ bool compile_pass(PassParam<R> &p, int n, int L, uint64_t T, const std::vector<I
         }
     }
     p.nruns = p.nops = p.npool = p.naux = 0;
-    std::vector<int> rest;
     while (!list.empty()) {
         if (p.nruns == kMaxRuns) return false;
         // first fit in order: a gate joins when its mixed bits fit the run and nothing it
@@ -802,7 +814,7 @@ bool compile_pass(PassParam<R> &p, int n, int L, uint64_t T, const std::vector<I
         uint64_t regs = 0, blocked = 0;
         RunDesc &rd = p.run[p.nruns++];
         const int first = p.nops;
-        std::vector<int> taken;
+        taken.clear();
         rest.clear();
         for (int g : list) {
             const Item &i = it[g];
@@ -1039,11 +1051,14 @@ template <typename R, int RP> struct Segment {
     int n, L, cmin, left;
     int K = 0;              // width of dense blocks, 0: none
     std::vector<int> list;  // the gates of the current pass, in a valid order
+    PlanScratch sc;
     uint64_t T = 0;         // its tile (PASS_RUNS, PASS_BLOCKS)
 
     Segment(const std::vector<Item> &items, const hq_gate *gs, int n_, int g0, int g1)
         : it(items), gates(gs), q(items, n_, g0, g1), n(n_), left(g1 - g0)
     {
+        list.reserve(size_t(left));
+        sc.reserve(size_t(left));
         tile_shape<R>(n, L, cmin);
         if (sizeof(R) == 4 && L >= kBlockTileMin) {
             if (n >= kBlockMinQubits) K = 3;
@@ -1097,7 +1112,7 @@ template <typename R, int RP> struct Segment {
             // the kind that does more work per time (work: what the gates cost in register runs)
             int head[HQ_MAX_N];
             std::memcpy(head, saved, sizeof(int) * size_t(n));
-            std::vector<int> blist;
+            std::vector<int> &blist = sc.blist;
             uint64_t btile = 0;
             grow(K, head, blist, btile);
             double runs = 0, work = 0;
@@ -1105,7 +1120,7 @@ template <typename R, int RP> struct Segment {
             for (int g : blist) work += run_cost(it[size_t(g)]);
             const double rate = list.empty() ? 0.0 : runs / std::max(kPassFloor, runs);
             if (!blist.empty() &&
-                work / std::max(kPassFloor, block_cost(K) * count_in_tile(n, K, gates, blist)) > rate) {
+                work / std::max(kPassFloor, block_cost(K) * count_in_tile(n, K, gates, blist, sc.block)) > rate) {
                 kind = PASS_BLOCKS;
                 list.swap(blist);
                 T = btile;
@@ -1135,7 +1150,7 @@ template <typename R, int RP> struct Segment {
         if (sizeof(R) == 4 && n >= 20) {
             double cost = runs, launches = 1;
             if (kind == PASS_BLOCKS) {
-                const int count = count_in_tile(n, K, gates, list), per = K == 3 ? kBlocks3 : kBlocks4;
+                const int count = count_in_tile(n, K, gates, list, sc.block), per = K == 3 ? kBlocks3 : kBlocks4;
                 launches = (count + per - 1) / per;
                 cost = block_cost(K) * count;
             }
@@ -1150,7 +1165,11 @@ template <typename R, int RP> struct Segment {
         // complex128 on up to 9 qubits: one CTA, a gate takes its FP64 latency (16 permutations of two qubits, n = 6 / 9: 83
         // / 80 us in runs, 66 in launches; two CNOT, n = 8: 10.6 and 8.2)
         if (sizeof(R) == 8 && n <= 9 && few_own <= 4.0 + few_run) kind = PASS_SINGLE;
-        while (kind == PASS_RUNS && !compile_pass<R, RP>(p, n, L, T, it, gates, list)) {
+        auto compiled = [&]() {
+            sc.todo = list;
+            return compile_pass<R, RP>(p, n, L, T, it, gates, sc);
+        };
+        while (kind == PASS_RUNS && !compiled()) {
             // too many runs: a shorter pass (the first half of the list is a valid order of its own)
             list.resize(list.size() / 2);
             std::memcpy(q.head, saved, sizeof(int) * size_t(n));
@@ -1170,7 +1189,6 @@ hq_status run_segment(void *state, int n, const std::vector<Item> &it, const hq_
     const hq_dtype dt = sizeof(R) == 4 ? HQ_C64 : HQ_C128;
     Segment<R, RP> seg(it, gates, n, g0, g1);
     PassParam<R> p;
-    std::vector<TileBlock> blocks;
     while (seg.left > 0) {
         hq_status st = HQ_OK;
         switch (seg.next(p)) {
@@ -1180,8 +1198,7 @@ hq_status run_segment(void *state, int n, const std::vector<Item> &it, const hq_
                     return st;
             break;
         case PASS_BLOCKS:
-            fuse_in_tile(n, seg.K, seg.T, gates, seg.list, blocks);
-            st = launch_block_pass(state, n, seg.L, seg.T, seg.K, blocks, s);
+            st = launch_block_pass(state, n, seg.L, seg.T, seg.K, gates, seg.list, seg.sc.block, s);
             break;
         default: {
             const size_t smem = pass_smem<R>(p.L);
