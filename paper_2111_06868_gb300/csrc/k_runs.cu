@@ -979,11 +979,11 @@ double block_cost(int K) { return K == 3 ? 0.39 : 0.77; }
 // permutation of four qubits 703 / 49 / 13 / 6.3, a dense four-qubit gate 860 / 59 / 16 / 8; controlled gates by what k_ctrl
 // touches: CNOT 376 / 21 / 7 / 4.3, a controlled SWAP 375 / 22 / 8.6 / 4.6, Toffoli 180-224 / 11-14 / 6.2 / 4.2, one with
 // three controls 145 / 9 / 7.5 / 7.4 (the last ones by the host).
-double own_time(const Item &i, int n)
+double own_time(const Item &i, double us_per_ms)
 {
     const double full = i.kind == OP_BLK && i.nb == 4 && !i.perm ? 0.86 : 0.69;
     const double ms = i.touched < 1.0 ? 0.04 + 0.63 * i.touched : full;  // n = 28
-    return std::max(4.2, 3.0 + std::ldexp(1e3 * ms, n - 28));
+    return std::max(4.2, 3.0 + us_per_ms * ms);
 }
 
 // complex128: the same for a gate in register runs and on its own kernel (ms at n = 28; FP64 multiply-adds at two per
@@ -1101,6 +1101,59 @@ template <typename R, int RP> struct Segment {
         for (int b = 0; b < n && __builtin_popcountll(tile) < L; ++b) tile |= uint64_t(1) << b;
     }
 
+    bool two_with_a_dense_one() const
+    {
+        return list.size() == 2 && (it[size_t(list[0])].kind == OP_U2 || it[size_t(list[1])].kind == OP_U2);
+    }
+
+    // Whether the gates of the pass in `list` are done sooner one launch each (estimated times).
+    bool own_kernels_faster(PassKind kind)
+    {
+        if (list.size() == 1) return true;
+        if constexpr (sizeof(R) == 4) {
+            // launches long enough to count: a list of Toffoli gates, n = 28, takes 0.41 ms each in blocks, 0.18 to 0.22 on
+            // k_ctrl.  A pass with little work in it does not hide all of that under its copies (n = 28: three CZ
+            // 0.87, three one-qubit gates 1.01, two Toffoli gates 1.03 ms).
+            if (n < 20) return false;
+            const double ms = std::ldexp(1e3, n - 28);  // us here of a ms at n = 28
+            double own = 0, cost = 0, launches = 1;
+            for (int g : list) {
+                const Item &i = it[size_t(g)];
+                own += own_time(i, ms);
+                // (a diagonal gate by its table: 0.185 of three qubits, 0.3 of six)
+                if (kind == PASS_RUNS) cost += i.kind == OP_DG ? 0.1 + 0.03 * i.nb : run_cost(i);
+            }
+            if (kind == PASS_BLOCKS) {
+                const int count = count_in_tile(n, K, gates, list, sc.block), per = K == 3 ? kBlocks3 : kBlocks4;
+                launches = (count + per - 1) / per;
+                cost = block_cost(K) * count;
+            }
+            return own <= kPassLaunch * launches + ms * std::max(cost, kPassFloor * launches + std::min(cost, 0.4));
+        } else if (n <= 9) {
+            // one CTA: a gate takes its FP64 latency (16 permutations of two qubits, n = 6 / 9: 83 / 80 us in runs, 66 in
+            // launches; two CNOT, n = 8: 10.6 and 8.2)
+            double own = 0, run = 4.0;
+            for (int g : list) {
+                const Item &i = it[size_t(g)];
+                own += i.kind == OP_U2 && i.keep == 0xffff ? 6.2 : 4.1;
+                run += i.kind == OP_U2 ? 4.9 : i.kind == OP_U1 && i.nb == 2 ? 3.3 : 1.0;
+            }
+            return own <= run || two_with_a_dense_one();
+        } else if (n < 17) {
+            return two_with_a_dense_one();
+        } else {
+            // where the FP64 work of the gates is what counts, a pass saves nothing (n >= 22: a pass of three CZ 2.4 at n =
+            // 24 and 2.6 at n = 26, the three on k_ctrl 2.0 and 1.7)
+            double own = 0, run = 0, light = 0;
+            for (int g : list) {
+                const Item &i = it[size_t(g)];
+                own += own_cost_128(i), run += run_cost_128(i);
+                light += i.kind == OP_PH && i.nb == 2 ? 0.3 : i.kind == OP_U1 && i.nb == 2 ? 0.55 : 1.0;
+            }
+            return (n >= 20 && light <= 1.0) || std::max(n >= 22 ? 2.4 : 1.3, run) >= 0.95 * own;
+        }
+    }
+
     // The next pass: register runs (into p), dense blocks (list and T), or single gates cheaper on their own kernels.
     PassKind next(PassParam<R> &p)
     {
@@ -1127,44 +1180,7 @@ template <typename R, int RP> struct Segment {
                 std::memcpy(q.head, head, sizeof(int) * size_t(n));
             }
         }
-        double own = 0, own64 = 0, run64 = 0, runs = 0, light = 0, few_own = 0, few_run = 0;
-        bool dense = false;
-        for (int g : list) {
-            const Item &i = it[size_t(g)];
-            own += own_time(i, n);
-            // (a diagonal gate by its table: 0.185 of three qubits, 0.3 of six)
-            runs += i.kind == OP_DG ? 0.1 + 0.03 * i.nb : run_cost(i);
-            dense = dense || i.kind == OP_U2;
-            if (sizeof(R) == 8) {
-                const bool full = i.kind == OP_U2 && i.keep == 0xffff;
-                few_own += full ? 6.2 : 4.1;
-                few_run += i.kind == OP_U2 ? 4.9 : i.kind == OP_U1 && i.nb == 2 ? 3.3 : 1.0;
-                own64 += own_cost_128(i), run64 += run_cost_128(i);
-                light += i.kind == OP_PH && i.nb == 2 ? 0.3 : i.kind == OP_U1 && i.nb == 2 ? 0.55 : 1.0;
-            }
-        }
-        if (list.size() == 1 || (sizeof(R) == 8 && n >= 20 && light <= 1.0)) kind = PASS_SINGLE;
-        // complex64, launches long enough to count: the pass only where it is the faster (a list of Toffoli gates, n =
-        // 28: 0.41 ms each in blocks, 0.18 to 0.22 on k_ctrl).  A pass with little work in it does not hide all of that
-        // under its copies (n = 28: three CZ 0.87, three one-qubit gates 1.01, two Toffoli gates 1.03 ms).
-        if (sizeof(R) == 4 && n >= 20) {
-            double cost = runs, launches = 1;
-            if (kind == PASS_BLOCKS) {
-                const int count = count_in_tile(n, K, gates, list, sc.block), per = K == 3 ? kBlocks3 : kBlocks4;
-                launches = (count + per - 1) / per;
-                cost = block_cost(K) * count;
-            }
-            const double pass = std::max(cost, kPassFloor * launches + std::min(cost, 0.4));
-            if (own <= kPassLaunch * launches + std::ldexp(1e3 * pass, n - 28)) kind = PASS_SINGLE;
-        }
-        // complex128: where the FP64 work of the gates is what counts, a pass saves nothing
-        // (n >= 22: a pass of three CZ 2.4 at n = 24 and 2.6 at n = 26, the three on k_ctrl 2.0 and 1.7)
-        if (sizeof(R) == 8 &&
-            (n >= 17 ? std::max(n >= 22 ? 2.4 : 1.3, run64) >= 0.95 * own64 : list.size() <= 2 && dense))
-            kind = PASS_SINGLE;
-        // complex128 on up to 9 qubits: one CTA, a gate takes its FP64 latency (16 permutations of two qubits, n = 6 / 9: 83
-        // / 80 us in runs, 66 in launches; two CNOT, n = 8: 10.6 and 8.2)
-        if (sizeof(R) == 8 && n <= 9 && few_own <= 4.0 + few_run) kind = PASS_SINGLE;
+        if (own_kernels_faster(kind)) kind = PASS_SINGLE;
         auto compiled = [&]() {
             sc.todo = list;
             return compile_pass<R, RP>(p, n, L, T, it, gates, sc);
