@@ -56,7 +56,8 @@ typedef int hq_status;
 #define HQ_ERR_DTYPE (-6)        /* unknown hq_dtype, or dtype not supported by the engine */
 #define HQ_ERR_ALLOC (-7)        /* device scratch (or host memory) allocation failed */
 #define HQ_ERR_CUDA (-8)         /* a CUDA runtime call failed */
-#define HQ_ERR_TIMEOUT (-9)      /* a bounded device-side wait ran out */
+#define HQ_ERR_TIMEOUT (-9)      /* a bounded device-side wait ran out (reported once, by the next synchronous call:
+                                    it waits for its own and for all blocking streams) */
 #define HQ_ERR_TOKEN (-10)       /* initial-state token not in {0,1,+,-} */
 #define HQ_ERR_CAPACITY (-11)    /* an output buffer is too small */
 #define HQ_ERR_ARG (-12)         /* any other invalid argument */

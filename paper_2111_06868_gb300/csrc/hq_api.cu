@@ -272,6 +272,20 @@ hq_status collect_result(const double *dev_value, double *out, DeviceFlags *flag
     FlagPtrs f;
     hq_status st = flag_ptrs(f);
     if (st != HQ_OK) return st;
+    // the flags are read after the work of every blocking stream, not only the call's own: on the legacy default stream,
+    // which waits for them (and, by an event, for a non-blocking s)
+    if (flags && s != nullptr && s != cudaStreamLegacy) {
+        unsigned kind = cudaStreamDefault;
+        if ((st = cuda_status("cudaStreamGetFlags", cudaStreamGetFlags(s, &kind))) != HQ_OK) return st;
+        if (kind & cudaStreamNonBlocking) {
+            const cudaEvent_t done = call_event();
+            if (!done) return HQ_ERR_ALLOC;
+            if ((st = cuda_status("record call event", cudaEventRecord(done, s))) != HQ_OK) return st;
+            if ((st = cuda_status("order the flags' read", cudaStreamWaitEvent(cudaStreamLegacy, done, 0))) != HQ_OK)
+                return st;
+        }
+        s = cudaStreamLegacy;
+    }
     CallResult *const r = call_result();
     if (!r) {  // no pinned memory: plain copies
         double v = 0;

@@ -273,10 +273,11 @@ struct DeviceFlags {
 // Synchronises s: the double at dev_value (NULL: none) into *out and the error
 // flags into *flags (NULL: not wanted), by one kernel that writes pinned host
 // memory -- one launch and one wait instead of a copy for the value and one for each flag.
+// With flags it also waits for the work already on the device's blocking streams, whose timeouts it reports.
 hq_status collect_result(const double *dev_value, double *out, DeviceFlags *flags, cudaStream_t s);
 // HQ_ERR_TIMEOUT (and clears the flags) if a bounded device-side wait ran out
 // since the last call: by what `flags` holds when it was read, else by reading
-// the flags after the work on s; synchronous.
+// the flags after the work on s and on all blocking streams; synchronous.
 hq_status device_error_status(cudaStream_t s, const DeviceFlags *flags = nullptr);
 // the same by plain copies, for callers that must not allocate (pinned memory included)
 hq_status device_error_status_plain();
