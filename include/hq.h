@@ -29,7 +29,9 @@
  *   - Threading: entry points may be called from several host threads; the
  *     per-device library state is set up once under a lock.
  *   - Device scratch: stream-ordered, from a memory pool that the library keeps
- *     per device (at most 16 MB stay mapped between calls).  Results of
+ *     per device: up to 16 MB of it stay mapped, what is above that is given back
+ *     at the first synchronisation after it was freed (a call that synchronises
+ *     frees before it waits; after one that does not, the caller's own).  Results of
  *     synchronous calls come back through a small pinned buffer per host thread.
  */
 #ifndef HQ_H

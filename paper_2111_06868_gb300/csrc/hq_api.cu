@@ -267,8 +267,19 @@ hq_status clear_flags(const FlagPtrs &f, const unsigned *v)
 }
 }  // namespace
 
-hq_status collect_result(const double *dev_value, double *out, DeviceFlags *flags, cudaStream_t s)
+hq_status collect_result(const double *dev_value, double *out, DeviceFlags *flags, cudaStream_t s, void *scratch)
 {
+    // freed before the wait, so that the pool can give back what it does not keep
+    struct Free {
+        void *p;
+        cudaStream_t on;
+        void now()
+        {
+            if (p) scratch_free(p, on);
+            p = nullptr;
+        }
+        ~Free() { now(); }
+    } held{scratch, s};
     FlagPtrs f;
     hq_status st = flag_ptrs(f);
     if (st != HQ_OK) return st;
@@ -284,19 +295,21 @@ hq_status collect_result(const double *dev_value, double *out, DeviceFlags *flag
             if ((st = cuda_status("order the flags' read", cudaStreamWaitEvent(cudaStreamLegacy, done, 0))) != HQ_OK)
                 return st;
         }
-        s = cudaStreamLegacy;
+        s = held.on = cudaStreamLegacy;
     }
     CallResult *const r = call_result();
     if (!r) {  // no pinned memory: plain copies
         double v = 0;
         if (dev_value)
             st = cuda_status("copy result", cudaMemcpyAsync(&v, dev_value, sizeof(v), cudaMemcpyDeviceToHost, s));
+        held.now();
         if (st == HQ_OK) st = cuda_status("sync", cudaStreamSynchronize(s));
         if (st == HQ_OK && dev_value && out) *out = v;
         return st;
     }
     k_collect<<<1, 32, 0, s>>>(dev_value, f, r);
     if ((st = cuda_status("k_collect", cudaGetLastError())) != HQ_OK) return st;
+    held.now();
     if ((st = cuda_status("sync", cudaStreamSynchronize(s))) != HQ_OK) return st;
     if (dev_value && out) *out = r->value;
     if (flags) {

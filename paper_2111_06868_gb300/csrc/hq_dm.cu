@@ -104,7 +104,7 @@ static hq_status run_dm_expectation(const void *rho, int n, const hq_pauli_term 
         k_dm_final<<<1, kDmThreads, 0, s>>>(scratch, nparts, scratch + nparts);
         st = cuda_status("k_dm_final", cudaGetLastError());
     }
-    if (st == HQ_OK) st = collect_result(scratch + nparts, out_host, nullptr, s);
+    if (st == HQ_OK) return collect_result(scratch + nparts, out_host, nullptr, s, scratch);
     scratch_free(scratch, s);
     return st;
 }

@@ -35,9 +35,10 @@ hq_status upload_async(void *dst, const void *src, size_t bytes, cudaStream_t s)
 // s made to wait for it: it does not queue behind the kernels already on s.
 hq_status upload_side(void *dst, const void *src, size_t bytes, cudaStream_t s, cudaEvent_t dst_ready);
 // Device scratch of a call: stream-ordered, from a pool that the library owns per
-// device (up to 16 MB stay mapped between calls: the default pool gives
-// everything back at each synchronisation, and mapping it again took 0.2 ms of a
-// call).  False when the memory cannot be had.
+// device (up to 16 MB stay mapped, more is given back at the first
+// synchronisation after it was freed: the default pool gives everything back
+// then, and mapping it again took 0.2 ms of a call).  False when the memory cannot
+// be had.
 bool scratch_alloc(void **p, size_t bytes, cudaStream_t s);
 void scratch_free(void *p, cudaStream_t s);
 // A per-thread, per-device event for one call's orderings (NULL on failure).
@@ -274,7 +275,9 @@ struct DeviceFlags {
 // flags into *flags (NULL: not wanted), by one kernel that writes pinned host
 // memory -- one launch and one wait instead of a copy for the value and one for each flag.
 // With flags it also waits for the work already on the device's blocking streams, whose timeouts it reports.
-hq_status collect_result(const double *dev_value, double *out, DeviceFlags *flags, cudaStream_t s);
+// scratch (NULL: none): the call's device scratch, which it frees, whatever it returns.
+hq_status collect_result(const double *dev_value, double *out, DeviceFlags *flags, cudaStream_t s,
+                         void *scratch = nullptr);
 // HQ_ERR_TIMEOUT (and clears the flags) if a bounded device-side wait ran out
 // since the last call: by what `flags` holds when it was read, else by reading
 // the flags after the work on s and on all blocking streams; synchronous.

@@ -674,7 +674,7 @@ hq_status launch_expectation(const void *state, int n, hq_dtype dt, const hq_pau
             if (injected_alloc_failure() || !scratch_alloc((void **)&scratch, sizeof(double) * nd, s))
                 return HQ_ERR_ALLOC;
             st = launch_tiled(state, n, dt, passes, grid, scratch, s);
-            if (st == HQ_OK) st = collect_result(scratch, out_host, flags, s);
+            if (st == HQ_OK) return collect_result(scratch, out_host, flags, s, scratch);
             scratch_free(scratch, s);
             return st;
         }
@@ -730,7 +730,7 @@ hq_status launch_expectation(const void *state, int n, hq_dtype dt, const hq_pau
         k_expect_final<<<1, kRedThreads, 0, s>>>(scratch, int(groups.size()), gx, scratch + npart);
         rc = cuda_status("k_expect_final", cudaGetLastError());
     }
-    if (rc == HQ_OK) rc = collect_result(scratch + npart, out_host, flags, s);
+    if (rc == HQ_OK) return collect_result(scratch + npart, out_host, flags, s, scratch);
     scratch_free(scratch, s);
     return rc;
 }
