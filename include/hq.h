@@ -29,7 +29,7 @@
  *   - Threading: entry points may be called from several host threads; the
  *     per-device library state is set up once under a lock.
  *   - Device scratch: stream-ordered, from a memory pool that the library keeps
- *     per device: up to 16 MB of it stay mapped, what is above that is given back
+ *     per device: up to 32 MB of it stay mapped, what is above that is given back
  *     at the first synchronisation after it was freed (a call that synchronises
  *     frees before it waits; after one that does not, the caller's own).  Results of
  *     synchronous calls come back through a small pinned buffer per host thread.

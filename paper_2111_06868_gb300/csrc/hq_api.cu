@@ -164,7 +164,9 @@ cudaEvent_t call_event()
 // device scratch
 // ----------------------------------------------------------------------------
 namespace {
-constexpr uint64_t kScratchKeep = 16 << 20;  // bytes a device's pool keeps mapped between calls
+// Bytes a device's pool keeps mapped between calls: one of the 32 MB pieces it grows by.  With less, a call that frees
+// its scratch before it waits gives its piece back each time and maps it again (hq_expectation 34 -> 185 us).
+constexpr uint64_t kScratchKeep = 32 << 20;
 
 cudaMemPool_t scratch_pool()
 {

@@ -35,7 +35,7 @@ hq_status upload_async(void *dst, const void *src, size_t bytes, cudaStream_t s)
 // s made to wait for it: it does not queue behind the kernels already on s.
 hq_status upload_side(void *dst, const void *src, size_t bytes, cudaStream_t s, cudaEvent_t dst_ready);
 // Device scratch of a call: stream-ordered, from a pool that the library owns per
-// device (up to 16 MB stay mapped, more is given back at the first
+// device (up to 32 MB stay mapped, more is given back at the first
 // synchronisation after it was freed: the default pool gives everything back
 // then, and mapping it again took 0.2 ms of a call).  False when the memory cannot
 // be had.

@@ -8,7 +8,7 @@ from paper_2111_06868_gb300 import circuits as C
 
 pytestmark = pytest.mark.gpu
 torch = pytest.importorskip("torch")
-KEPT = 16 << 20  # what the pool keeps mapped
+KEPT = 32 << 20  # what the pool keeps mapped
 SLACK = 4 << 20  # other users of the device memory in this process
 
 
