@@ -32,7 +32,8 @@
  *     per device: up to 32 MB of it stay mapped, what is above that is given back
  *     at the first synchronisation after it was freed (a call that synchronises
  *     frees before it waits; after one that does not, the caller's own).  Results of
- *     synchronous calls come back through a small pinned buffer per host thread.
+ *     synchronous calls come back through small pinned buffers, as many as calls
+ *     have run at the same time.
  */
 #ifndef HQ_H
 #define HQ_H

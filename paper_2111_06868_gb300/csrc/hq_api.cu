@@ -245,18 +245,64 @@ hq_status flag_ptrs(FlagPtrs &f)
     return HQ_OK;
 }
 
-// pinned, one per host thread and device (like the staging ring); NULL on failure
-CallResult *call_result()
+// Pinned result buffers (with an event): taken for a call and given back, so as many as calls have run at the same time
+// (one per host thread would stay behind when the thread ends).
+struct CallRecord {
+    CallResult *host = nullptr;
+    cudaEvent_t done = nullptr;
+};
+struct RecordPool {
+    std::mutex mu;
+    std::vector<CallRecord> idle[64];
+};
+RecordPool &record_pool()
 {
-    static thread_local CallResult *r[64] = {nullptr};
-    int dev = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return nullptr;
-    if (!r[dev] && cudaHostAlloc((void **)&r[dev], sizeof(CallResult), cudaHostAllocDefault) != cudaSuccess) {
-        cudaGetLastError();
-        r[dev] = nullptr;
-    }
-    return r[dev];
+    static RecordPool *const pool = new RecordPool;  // never destroyed: calls may still run while the process ends
+    return *pool;
 }
+class BorrowedRecord {
+  public:
+    // host() and done(): NULL where they cannot be had
+    BorrowedRecord()
+    {
+        if (cudaGetDevice(&dev_) != cudaSuccess || dev_ < 0 || dev_ >= 64) return;
+        {
+            std::lock_guard<std::mutex> lk(record_pool().mu);
+            std::vector<CallRecord> &idle = record_pool().idle[dev_];
+            if (!idle.empty()) {
+                r_ = idle.back();
+                idle.pop_back();
+                return;
+            }
+        }
+        if (cudaHostAlloc((void **)&r_.host, sizeof(CallResult), cudaHostAllocDefault) != cudaSuccess) {
+            cudaGetLastError();
+            r_.host = nullptr;
+        } else if (cudaEventCreateWithFlags(&r_.done, cudaEventDisableTiming) != cudaSuccess) {
+            cudaGetLastError();
+            r_.done = nullptr;
+        }
+    }
+    ~BorrowedRecord()
+    {
+        if (!r_.host) return;
+        try {
+            std::lock_guard<std::mutex> lk(record_pool().mu);
+            record_pool().idle[dev_].push_back(r_);
+        } catch (const std::bad_alloc &) {
+            cudaFreeHost(r_.host);
+            if (r_.done) cudaEventDestroy(r_.done);
+        }
+    }
+    BorrowedRecord(const BorrowedRecord &) = delete;
+    CallResult *host() const { return r_.host; }
+    cudaEvent_t done() const { return r_.done; }
+    void forget() { r_ = CallRecord(); }  // (a kernel may still write it)
+
+  private:
+    int dev_ = 0;
+    CallRecord r_;
+};
 
 hq_status clear_flags(const FlagPtrs &f, const unsigned *v)
 {
@@ -285,21 +331,22 @@ hq_status collect_result(const double *dev_value, double *out, DeviceFlags *flag
     FlagPtrs f;
     hq_status st = flag_ptrs(f);
     if (st != HQ_OK) return st;
+    BorrowedRecord record;
     // the flags are read after the work of every blocking stream, not only the call's own: on the legacy default stream,
     // which waits for them (and, by an event, for a non-blocking s)
     if (flags && s != nullptr && s != cudaStreamLegacy) {
         unsigned kind = cudaStreamDefault;
         if ((st = cuda_status("cudaStreamGetFlags", cudaStreamGetFlags(s, &kind))) != HQ_OK) return st;
         if (kind & cudaStreamNonBlocking) {
-            const cudaEvent_t done = call_event();
-            if (!done) return HQ_ERR_ALLOC;
-            if ((st = cuda_status("record call event", cudaEventRecord(done, s))) != HQ_OK) return st;
-            if ((st = cuda_status("order the flags' read", cudaStreamWaitEvent(cudaStreamLegacy, done, 0))) != HQ_OK)
-                return st;
+            st = record.done() ? cuda_status("record call event", cudaEventRecord(record.done(), s))
+                               : cuda_status("sync", cudaStreamSynchronize(s));
+            if (st == HQ_OK && record.done())
+                st = cuda_status("order the flags' read", cudaStreamWaitEvent(cudaStreamLegacy, record.done(), 0));
+            if (st != HQ_OK) return st;
         }
         s = held.on = cudaStreamLegacy;
     }
-    CallResult *const r = call_result();
+    CallResult *const r = record.host();
     if (!r) {  // no pinned memory: plain copies
         double v = 0;
         if (dev_value)
@@ -312,7 +359,10 @@ hq_status collect_result(const double *dev_value, double *out, DeviceFlags *flag
     k_collect<<<1, 32, 0, s>>>(dev_value, f, r);
     if ((st = cuda_status("k_collect", cudaGetLastError())) != HQ_OK) return st;
     held.now();
-    if ((st = cuda_status("sync", cudaStreamSynchronize(s))) != HQ_OK) return st;
+    if ((st = cuda_status("sync", cudaStreamSynchronize(s))) != HQ_OK) {
+        record.forget();
+        return st;
+    }
     if (dev_value && out) *out = r->value;
     if (flags) {
         flags->read = true;
