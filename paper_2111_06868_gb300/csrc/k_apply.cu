@@ -437,8 +437,8 @@ __device__ __forceinline__ void tiles_pipelined(const TileGeom &g, float2 *__res
     cp_async_wait<0>();
 }
 
-// The same for kernels that the issue slots bound, tiles of 2^g.L <= 2^LB
-// amplitudes and TH >= 128 threads: a thread's copies lie 2 TH amplitudes
+// The same for kernels that the issue slots bound, tiles of 2^LB amplitudes
+// (g.L = LB: states of at least LB qubits) and TH >= 128 threads: a thread's copies lie 2 TH amplitudes
 // apart, above the bits the swizzle reads, so each address is the thread's
 // first one plus an offset that all threads share (from shared memory in the
 // state, an immediate in the tile).  Per-copy addresses cost the K = 4 kernel
@@ -454,43 +454,37 @@ __device__ __forceinline__ void tiles_pipelined_lean(const TileGeom &g, float2 *
     float2 *const buf = reinterpret_cast<float2 *>(smem_raw);
     const int TS = 1 << g.L, cmask = (1 << g.c) - 1;
     const int first = int(threadIdx.x) * 2, f = (first >> 4) & 15;
-    const bool copier = first < TS;
-    if (threadIdx.x < NC && int(threadIdx.x) * STEP < TS) {
+    if (threadIdx.x < NC) {
         const int i = int(threadIdx.x) * STEP;
         s_k[threadIdx.x] = g.runoff[i >> g.c] + (i & cmask);
     }
-    const int64_t off = copier ? g.runoff[first >> g.c] + (first & cmask) : 0;
+    const int64_t off = g.runoff[first >> g.c] + (first & cmask);
     __syncthreads();
-    const bool full = g.L == LB;  // (smaller only for states of fewer than LB qubits: one tile)
-    // both loops free of conditions when the tile is full: the loads of all copies overlap
+    // both loops free of per-copy conditions: the loads of all copies overlap.  (`full` always holds; without the test
+    // the compiler orders the copies so that the kernel takes 0.93 instead of 0.86 ms at n = 28.)
+    const bool full = g.L == LB;
     auto load = [&](int64_t t, float2 *to) {
         const float2 *const src = state + tile_base(g, t) + off;
-        auto copy = [&](int k) {
-            if (f & 1) {
-                cp_async8(to + (first ^ f) + k * STEP, src + s_k[k]);
-                cp_async8(to + ((first + 1) ^ f) + k * STEP, src + s_k[k] + 1);
-            } else {
-                cp_async16(to + (first ^ f) + k * STEP, src + s_k[k]);
-            }
-        };
         if (full) {
 #pragma unroll
-            for (int k = 0; k < NC; ++k) copy(k);
-        } else if (copier) {
-            for (int k = 0; k * STEP < TS; ++k) copy(k);
+            for (int k = 0; k < NC; ++k) {
+                if (f & 1) {
+                    cp_async8(to + (first ^ f) + k * STEP, src + s_k[k]);
+                    cp_async8(to + ((first + 1) ^ f) + k * STEP, src + s_k[k] + 1);
+                } else {
+                    cp_async16(to + (first ^ f) + k * STEP, src + s_k[k]);
+                }
+            }
         }
     };
     auto store = [&](int64_t t, const float2 *from) {
         float2 *const dst = state + tile_base(g, t) + off;
-        auto copy = [&](int k) {
-            const float4 w = *reinterpret_cast<const float4 *>(from + ((first ^ f) & ~1) + k * STEP);
-            *reinterpret_cast<float4 *>(dst + s_k[k]) = (f & 1) ? make_float4(w.z, w.w, w.x, w.y) : w;
-        };
         if (full) {
 #pragma unroll
-            for (int k = 0; k < NC; ++k) copy(k);
-        } else if (copier) {
-            for (int k = 0; k * STEP < TS; ++k) copy(k);
+            for (int k = 0; k < NC; ++k) {
+                const float4 w = *reinterpret_cast<const float4 *>(from + ((first ^ f) & ~1) + k * STEP);
+                *reinterpret_cast<float4 *>(dst + s_k[k]) = (f & 1) ? make_float4(w.z, w.w, w.x, w.y) : w;
+            }
         }
     };
     int64_t t = blockIdx.x;
@@ -982,52 +976,61 @@ static hq_status run_mono(void *state, int n, const int *qubits, const double *m
     return cuda_status("k_mono", cudaGetLastError());
 }
 
+static_assert(kPairMinQubits >= kPairTileBits, "tiles_pipelined_lean takes full tiles only");
+template <int K>
+static hq_status run_gather_pair(void *state, int n, const int *qubits, const double *mat, int64_t nstates,
+                                 cudaStream_t s)
+{
+    TileGeom g;
+    make_geom(g, n, K, qubits, std::min(n, kPairTileBits), nstates);
+    PairMatParam<K> p;
+    for (int r = 0; r < (1 << K); ++r) {
+        p.off[r] = (g.toff[r] ^ ((g.toff[r] >> 4) & 15)) * int(sizeof(float2));
+        for (int c = 0; c < (1 << K); ++c) {
+            const double *e = mat + 2 * (r * (1 << K) + c);
+            const float re[2] = {float(e[0]), float(e[0])}, im[2] = {float(e[1]), float(e[1])};
+            std::memcpy(&p.a[r][c].x, re, 8);
+            std::memcpy(&p.a[r][c].y, im, 8);
+        }
+    }
+    const size_t smem = size_t(2 * sizeof(float2)) << g.L;
+    const void *fn = (const void *)k_gather_pair<K>;
+    const int grid = grid_for(fn, kPairThreads, smem, g.total_tiles);
+    k_gather_pair<K><<<grid, kPairThreads, smem, s>>>(g, p, (float2 *)state);
+    return cuda_status("k_gather_pair", cudaGetLastError());
+}
+
 template <typename R, int K>
 static hq_status run_gather(void *state, int n, const int *qubits, const double *mat, int64_t nstates, cudaStream_t s)
 {
-    TileGeom g;
-    make_geom(g, n, K, qubits, tile_bits<R>(n), nstates);
-    MatParam<R, K> m;
-    for (int r = 0; r < (1 << K); ++r)
-        for (int c = 0; c < (1 << K); ++c) {
-            m.a[r][c].x = R(mat[2 * (r * (1 << K) + c)]);
-            m.a[r][c].y = R(mat[2 * (r * (1 << K) + c) + 1]);
-        }
-    // complex64: the next tile's load in flight under the current one (two buffers per CTA)
-    if constexpr (sizeof(R) == 4 && K >= 3) {
-        if (K == 3 || n >= kPairMinQubits) {
-            make_geom(g, n, K, qubits, std::min(n, kPairTileBits), nstates);
-            PairMatParam<K> p;
-            for (int r = 0; r < (1 << K); ++r) {
-                p.off[r] = (g.toff[r] ^ ((g.toff[r] >> 4) & 15)) * int(sizeof(float2));
-                for (int c = 0; c < (1 << K); ++c) {
-                    const float2 re = make_float2(m.a[r][c].x, m.a[r][c].x), im = make_float2(m.a[r][c].y, m.a[r][c].y);
-                    std::memcpy(&p.a[r][c].x, &re, 8);
-                    std::memcpy(&p.a[r][c].y, &im, 8);
-                }
+    if constexpr (sizeof(R) == 4 && K == 3) {
+        return run_gather_pair<K>(state, n, qubits, mat, nstates, s);
+    } else {
+        if constexpr (sizeof(R) == 4 && K == 4)
+            if (n >= kPairMinQubits) return run_gather_pair<K>(state, n, qubits, mat, nstates, s);
+        TileGeom g;
+        make_geom(g, n, K, qubits, sizeof(R) == 4 ? std::min(n, 11) : tile_bits<R>(n), nstates);
+        MatParam<R, K> m;
+        for (int r = 0; r < (1 << K); ++r)
+            for (int c = 0; c < (1 << K); ++c) {
+                m.a[r][c].x = R(mat[2 * (r * (1 << K) + c)]);
+                m.a[r][c].y = R(mat[2 * (r * (1 << K) + c) + 1]);
             }
+        if constexpr (sizeof(R) == 4) {
+            // the next tile's load in flight under the current one (two buffers per CTA)
             const size_t smem = size_t(2 * sizeof(float2)) << g.L;
-            const void *fn = (const void *)k_gather_pair<K>;
-            const int grid = grid_for(fn, kPairThreads, smem, g.total_tiles);
-            k_gather_pair<K><<<grid, kPairThreads, smem, s>>>(g, p, (float2 *)state);
-            return cuda_status("k_gather_pair", cudaGetLastError());
+            const void *fn = (const void *)k_gather_pipe<K>;
+            const int grid = grid_for(fn, kThreads, smem, g.total_tiles);
+            k_gather_pipe<K><<<grid, kThreads, smem, s>>>(g, m, (float2 *)state);
+            return cuda_status("k_gather_pipe", cudaGetLastError());
+        } else {
+            const size_t smem = size_t(sizeof(typename C2<R>::type)) << g.L;
+            const void *fn = (const void *)k_gather<R, K>;
+            const int grid = grid_for(fn, kThreads, smem, g.total_tiles);
+            k_gather<R, K><<<grid, kThreads, smem, s>>>(g, m, (typename C2<R>::type *)state);
+            return cuda_status("k_gather", cudaGetLastError());
         }
     }
-    if constexpr (sizeof(R) == 4 && K != 3) {
-        make_geom(g, n, K, qubits, std::min(n, 11), nstates);
-        const size_t smem = size_t(2 * sizeof(float2)) << g.L;
-        const void *fn = (const void *)k_gather_pipe<K>;
-        const int grid = grid_for(fn, kThreads, smem, g.total_tiles);
-        k_gather_pipe<K><<<grid, kThreads, smem, s>>>(g, m, (float2 *)state);
-        return cuda_status("k_gather_pipe", cudaGetLastError());
-    } else if constexpr (sizeof(R) == 8) {
-        const size_t smem = size_t(sizeof(typename C2<R>::type)) << g.L;
-        const void *fn = (const void *)k_gather<R, K>;
-        const int grid = grid_for(fn, kThreads, smem, g.total_tiles);
-        k_gather<R, K><<<grid, kThreads, smem, s>>>(g, m, (typename C2<R>::type *)state);
-        return cuda_status("k_gather", cudaGetLastError());
-    }
-    return HQ_OK;  // (not reached: complex64 K = 3 always takes k_gather_pair)
 }
 
 template <typename R, int K>
