@@ -444,9 +444,14 @@ hq_status hq_apply_gate(void *state, int n, hq_dtype dt, const int *qubits, int 
  * diagonal gates (complex64: of up to 4 qubits) many at a time, each tile of the
  * state read and written once per pass (gates with disjoint qubits may swap; on
  * large complex64 states a pass's gates are multiplied, in double, into blocks of 3 or
- * 4 qubits first); a product with an exactly zero real or imaginary part of a
- * matrix entry may be left out there, so an infinity or NaN among the amplitudes
- * may spread only through nonzero parts.
+ * 4 qubits first, unless a product leaves single precision's range); a pass is
+ * used where it is estimated to be faster than one launch per gate.
+ * An infinity or NaN among the amplitudes is not lost there (as long as no gate
+ * has an all-zero column), but the amplitudes that it spreads to are not those of
+ * one gate at a time: products with an exactly zero real or imaginary part of a
+ * matrix entry may be left out (it spreads to fewer), and a block multiplies by its
+ * exact zeros (it spreads to every amplitude that differs in the block's qubits only,
+ * among them, where a block is widened, qubits that no gate acts on).
  * Errors: as hq_apply_gate, plus HQ_ERR_ARG (G < 0 or unknown engine).
  * On HQ_ERR_ALLOC the state is left as follows: the tensor-core engines and
  * HQ_ENGINE_TC_PASS take their one scratch buffer before enqueueing any

@@ -90,3 +90,35 @@ def test_lists_of_controlled_gates(hq, n, form):
     # exact products but for the sums of zeros and the order of disjoint gates: the same amplitudes
     assert float(torch.linalg.norm(st - one)) <= 2e-6 * float(torch.linalg.norm(one))
     assert time([gates]) <= 1.5 * time(singles)
+
+
+@pytest.mark.parametrize("dtype", ["complex64", "complex128"])
+@pytest.mark.parametrize("n", [5, 9, 12, 20, 23])
+@pytest.mark.parametrize("bad", [float("nan"), float("inf"), complex(0, float("inf"))])
+def test_infinities_and_nan(hq, n, dtype, bad):
+    """One amplitude that is not finite: never lost by gates without a zero
+    column; without blocks, amplitudes that differ in a qubit no gate acts on
+    are those of the state without it."""
+    sm, rng = C.SplitMix64(n), np.random.default_rng(n)
+    forms = [lambda: (1, C.hadamard()), lambda: (1, C.sqrt_x()), lambda: (1, C.PAULI["Y"]), lambda: (2, C.cnot()),
+             lambda: (2, C.cz()), lambda: (2, C.swap()), lambda: (2, C.fsim(np.pi / 2, 0.3)),
+             lambda: (2, C.random_unitary(2, sm)), lambda: (1, np.diag(np.exp(1j * rng.uniform(0, 6, 2))))]
+    act = n - 2  # qubits 0 .. n - 3 only
+    gates = []
+    for _ in range(40):
+        k, m = forms[rng.integers(len(forms))]()
+        gates.append(C.Gate("a", tuple(int(q) for q in rng.choice(act, k, replace=False)), m))
+    st = torch.randn(1 << n, dtype=getattr(torch, dtype), device="cuda") * 2.0 ** (-n / 2)
+    at = int(rng.integers(1 << n))
+    st[at] = 0
+    clean = st.clone()
+    st[at] = bad
+    hq.hq_apply_blocks(clean, gates)
+    hq.hq_apply_blocks(st, gates)
+    finite = torch.isfinite(torch.view_as_real(st)).all(dim=1)
+    assert not bool(finite.all())
+    assert not np.isfinite(hq.hq_expectation(st, [(1.0, ())]))
+    if n < 23 or dtype == "complex128":
+        apart = (torch.arange(1 << n, device="cuda") ^ at) & 3 != 0  # the two lowest bits: qubits n - 2, n - 1
+        assert bool(finite[apart].all())
+        assert torch.equal(torch.view_as_real(st[apart]), torch.view_as_real(clean[apart]))
