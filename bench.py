@@ -161,7 +161,7 @@ def measured_traffic(kernel_class, n):
 
 
 def block_class(qs, m, engine, tc_min_k, n=30, elem_bytes=8):
-    """Which kernel libhq launches for this block (mirrors its dispatch:
+    """Which kernel libhq launches for this block on its own (mirrors its dispatch:
     controlled gates first, tensor-core blocks of k = 4, 5 run widened to 6
     qubits when n >= 13)."""
     from paper_2111_06868_gb300 import hq
@@ -187,19 +187,6 @@ def block_class(qs, m, engine, tc_min_k, n=30, elem_bytes=8):
     if engine in ("df", "tc_c128") and elem_bytes == 16 and k <= 4:
         return f"k_gather_df_k{k}"
     return f"k_gather_k{k}" if k <= 4 else f"k_block_k{k}"
-
-
-def touched_fraction(qs, m, n, elem_bytes):
-    """Fraction of the state's bytes one gate reads and writes: 2^-c for the
-    controlled-gate kernel with c controls at or above the 32-byte sector,
-    else 1."""
-    from paper_2111_06868_gb300 import hq
-
-    if not block_class(qs, m, "auto", 4, n, elem_bytes).startswith("k_ctrl"):
-        return 1.0
-    _, mask, _ = hq.hq_gate_structure(m)
-    sector_bits = 2 if elem_bytes == 8 else 1
-    return 2.0 ** -sum(1 for j, q in enumerate(qs) if (mask >> j) & 1 and n - 1 - q >= sector_bits)
 
 
 def cpu_model() -> str:
@@ -323,8 +310,8 @@ def _time_blocks(n, blocks, engine, dtype, reps=1, tc_min_k=4):
 
 
 def measure_small_circuit(args, reps: int = 20):
-    """One small circuit (n=12, 163 gates; latency-bound): per-block launches
-    of the fused circuit against one persistent launch of the batch runner."""
+    """One small circuit (n=12, 163 gates; latency-bound): the fused circuit
+    through hq_apply_blocks against one persistent launch of the batch runner."""
     import torch
     from paper_2111_06868_gb300 import hq
 
@@ -506,14 +493,15 @@ def measure_fp_peaks(N=8192, reps=5):
 def measure_c128(args, circ):
     """Configuration 2 in complex128: per gate and fused k <= 4 on the FP64
     kernels, in double-float, and fused k <= 3, 4 on the tensor cores (exact
-    digit-slice products); rates in unfused gate-apps/s, effective GB/s =
-    bytes of one read and write of the state per launch."""
+    digit-slice products); rates in unfused gate-apps/s; GB/s where every
+    gate or block is a launch of its own = bytes of one read and write of the
+    state per launch."""
     import torch
 
     G = len(circ.gates)
     res = {"gates": G}
     st, t = _time_blocks(30, [(g.qubits, g.matrix) for g in circ.gates], "auto", torch.complex128)
-    res["per_gate"] = {"launches": G, "gate_apps_per_s": G / t, "s": t, "GBps": G * 2 * (1 << 30) * 16 / t / 1e9}
+    res["per_gate"] = {"gates": G, "gate_apps_per_s": G / t, "s": t}
     del st
     from paper_2111_06868_gb300 import hq
 
@@ -594,14 +582,14 @@ def measure_extras(args):
     from paper_2111_06868_gb300 import hq
 
     out = {}
-    # n=30, unfused: every gate its own launch
+    # n=30, unfused gates, on the exact engine (which takes several per pass over the state)
     circ = C.config_n30(seed=args.seed)
     G = len(circ.gates)
     st, t = _time_blocks(30, [(g.qubits, g.matrix) for g in circ.gates], "auto", torch.complex64)
-    out["n30_per_gate_c64"] = {"gate_apps_per_s": G / t, "s": t, "launches": G}
+    out["n30_per_gate_c64"] = {"gate_apps_per_s": G / t, "s": t, "gates": G}
     del st
     # the same circuit fused into blocks of <= 4 qubits on the exact FP32
-    # CUDA-core kernels (gather / monomial / diagonal; no tensor cores)
+    # CUDA-core kernels (passes of several blocks; no tensor cores)
     b4 = fuse(hq, 30, circ.gates, 4, args)
     st, t4 = _time_blocks(30, b4, "cuda_core", torch.complex64)
     out["n30_fused_k4_c64_cuda_core"] = {"blocks": len(b4), "gate_apps_per_s": G / t4, "s": t4,
@@ -611,15 +599,11 @@ def measure_extras(args):
     # <= 4-qubit blocks on the exact kernels
     out["n30_c128"] = measure_c128(args, circ)
     torch.cuda.empty_cache()
-    # n=30 QFT, unfused: 435 controlled phases (the controlled-gate kernel reads
-    # and writes only the amplitudes whose controls are 1), 30 H, 15 SWAP
+    # n=30 QFT, unfused: 435 controlled phases, 30 H, 15 SWAP in passes
     qft = [(g.qubits, g.matrix) for g in C.qft_circuit(30).gates]
-    for name, dt, S in (("c64", torch.complex64, 8), ("c128", torch.complex128, 16)):
+    for name, dt in (("c64", torch.complex64), ("c128", torch.complex128)):
         st, t = _time_blocks(30, qft, "auto", dt)
-        touched = sum(touched_fraction(q, m, 30, S) for q, m in qft) * 2 * (1 << 30) * S
-        out[f"n30_qft_per_gate_{name}"] = {"gates": len(qft), "gate_apps_per_s": len(qft) / t, "s": t,
-                                           "touched_GBps": touched / t / 1e9,
-                                           "full_pass_equivalents": touched / (2 * (1 << 30) * S)}
+        out[f"n30_qft_per_gate_{name}"] = {"gates": len(qft), "gate_apps_per_s": len(qft) / t, "s": t}
         del st
         torch.cuda.empty_cache()
     # n=30 <Z_0> after the circuit: Sec. 3.1 pop (light cone of qubit 0) and
@@ -1100,7 +1084,11 @@ def main():
         last_tc = classes[-1].startswith("k_tc") or (engine in ("tc_f16", "tc_bf16") and n >= 13 and
                                                      4 <= len(blocks[-1][0]) <= 6)
         passes_rw = 2 * B - (1 if first_tc else -1) + (0 if last_tc else 1)
-        eff_gbs = passes_rw * (bytes_per_launch // 2) * args.steps / (elapsed / world) / 1e9
+        # (the exact engines take several blocks per pass: no count of their reads and writes here, and a count of
+        # launches that is only a lower bound, one for each block that a pass does not take)
+        in_passes = engine in ("auto", "cuda_core")
+        launches = B if not in_passes else sum(len(q) > 4 for q, _ in blocks) + any(len(q) <= 4 for q, _ in blocks)
+        eff_gbs = None if in_passes else passes_rw * (bytes_per_launch // 2) * args.steps / (elapsed / world) / 1e9
         rec = {
             "metric": METRIC, "value": value, "unit": "gate-apps/s", "n_gpus": world, "steps": args.steps,
             "warmup": args.warmup, "ms_per_step": 1e3 * elapsed / args.steps, "higher_is_better": True,
@@ -1119,7 +1107,7 @@ def main():
                               else f"state ({S << n} B) fits in L2 and is not flushed"),
                        "parallelism": f"replicas x{world}" if world > 1 else "single GPU",
                        **({"passes": passes} if engine == "tc_pass" else {})},
-            "effective_GBps": eff_gbs, "roofline_frac_effective": eff_gbs / peaks["hbm_gbs"],
+            "effective_GBps": eff_gbs, "roofline_frac_effective": eff_gbs and eff_gbs / peaks["hbm_gbs"],
             "roofline": {"bound": "hbm", "achieved": achieved, "peak": peaks["hbm_gbs"], "unit": "GB/s",
                          "frac": achieved / peaks["hbm_gbs"], "traffic": measured_traffic(dom, n),
                          "kernel": dom, "peak_source": peak_kind,
@@ -1127,8 +1115,8 @@ def main():
             "per_class": per_class,
             "norm2": norm, "fuse_s": fuse_s, "per_block_pass_ms_per_step": 1e3 * per_block_step_s,
             "e2e": e2e, "cpu_baseline": cpu, "clocks": clocks, "extras": extras,
-            # per step: the blocks, k_init unless folded, the norm (k_expect + k_expect_final) unless folded
-            "gpu_launches": args.steps * (B + (0 if first_tc else 1) + (0 if last_tc else 2)),
+            # per step: the blocks, k_init unless folded, the norm (k_expect + k_expect_final) unless folded, k_collect
+            "gpu_launches": args.steps * (launches + (0 if first_tc else 1) + (0 if last_tc else 2) + 1),
         }
         print(json.dumps(rec))
     if dist:
