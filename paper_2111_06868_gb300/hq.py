@@ -185,7 +185,7 @@ def _stream(stream):
 
 
 def _data_ptr(a: np.ndarray) -> int:
-    return a.__array_interface__["data"][0]
+    return a.ctypes.data
 
 
 # one record of each C struct by its number of qubits (native alignment): a whole struct per call instead of one
@@ -528,15 +528,16 @@ def hq_expectation_static(state, H, stream=None) -> float:
 
 def _ops_array(circuit, keep: list):
     arr = (hq_op * max(1, len(circuit.gates)))()
-    known: dict = {}
     for i, g in enumerate(circuit.gates):
         op = arr[i]
         op.k = g.k
         for j, q in enumerate(g.qubits):
             op.qubits[j] = int(q)
         if g.matrix is not None:
+            m = np.ascontiguousarray(g.matrix, np.complex128)
+            keep.append(m)
             op.kind = HQ_OP_MATRIX
-            op.matrix = _matrix_ptr(g.matrix, known, keep)
+            op.matrix = m.ctypes.data
         else:
             op.kind = HQ_OP_ROT
             op.axis = ord(g.axis)
