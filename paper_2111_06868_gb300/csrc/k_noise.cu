@@ -445,10 +445,10 @@ static hq_status sample_on_device(void *state, int n, const int *qubits, PickArg
 // write of the state instead of a read, a one-CTA pick and a read and write.
 // A thread holds 16 amplitudes: all values of this window's two qubits and of
 // the next one's (a qubit that a window lacks is replaced by any other bit).
-// Bound: HBM (two channels at n = 24: 268 MB, 40 us at the copy bandwidth; the
-// launch takes 67-73 us with cold caches, where three launches per channel took
-// 101), with about 5 us of FP64 latency per launch for the pick; complex128 the
-// FP64 pipe.
+// Bound: HBM (two channels at n = 24: 268 MB, 40 us at the copy bandwidth; a
+// launch takes 74 us, the mean of a trajectory's 156 serialised ones, where
+// three launches per channel took 101), with about 5 us of FP64 latency per
+// launch for the pick; complex128 the FP64 pipe.
 // ----------------------------------------------------------------------------
 constexpr int kWindowRow = 20;  // sums per CTA: 10 complex entries of the upper triangle
 struct WindowParam {

@@ -29,7 +29,8 @@
 // Tried and slower, n=28 circuit (785 gates): 8 amplitudes per thread 123 ms, scalar FMAs 120 ms, packed real and
 // scalar imaginary products 94 ms, 512 threads at 64 registers 102 ms, two CTAs per SM 95 ms, against 87 ms.
 // From 23 qubits on (and for 3- and 4-qubit gates) a complex64 pass may instead fuse its gates into dense blocks
-// (k_block_pass.cu); the kind that does more work per time is chosen pass by pass.
+// (k_block_pass.cu); the kind that does more work per time is chosen pass by pass, and the gates' own kernels where their
+// estimated time is below that of the pass (own_kernels_faster).
 // Per-gate circuits, against one launch per gate: n=28 complex64 depth 20 fSim 528 -> 87 ms (55 in blocks), n=20
 // depth 16 CZ 1.53 -> 0.25 ms of device time, n=12 complex128 depth 10 1.06 -> 0.20 ms.
 #include <algorithm>
